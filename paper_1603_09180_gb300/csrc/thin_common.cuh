@@ -146,10 +146,71 @@ constexpr PointTable make_point_table(int adj)
 constexpr PointTable kPointTable = make_point_table(0);
 constexpr PointTable kPointTable48 = make_point_table(1);
 
-// Shared-memory table block of every kernel: the point table of (8,4), then
-// that of (4,8), 256 words each.
-constexpr int kTabWords = 512;
-constexpr int kTabOffset48 = 256;
+// The decision of Sec. 2.1 and 2.2 for every state of the eight neighbours.  In
+// every mode it depends on the pixel values through two masks only: the
+// neighbours below F(x), and those of them below F(x) - lambda ("deep").  So a
+// neighbour has one of three states, t = 0 (not lower), 1 (lower, at least
+// F(x) - lambda) or 2 (deep), and the entry of the ring's states is
+// v[sum t_d 3^d]: bit m is set where a point may be lowered in mode m (bit 0 of
+// the mode: the F^- reading, bit 1: the operator, bit 2: the adjacency pair).
+// 6561 bytes serve every mode, which one bit per pair of masks (8 KiB a mode)
+// would not.  At lambda = 0 every lower neighbour is deep.
+constexpr int kDecisions = 6561;
+constexpr int kDecisionBytes = 6576;  // padded to whole 16-byte vectors
+
+struct DecisionTable {
+    alignas(16) uint8_t v[kDecisionBytes];
+};
+
+// Whether a point with lower neighbours `lower`, of which `deep` are below
+// F(x) - lambda, may be lowered (e: its entry in the pair's point table).
+// A k-divergent point needs at least k - 1 components c with
+// F(x) - F^-(c) <= lambda; F^- is the largest (rule 0: one shallow member is
+// enough) or the smallest value over c (rule 1: no member may be deep).
+constexpr bool decision(uint32_t e, unsigned lower, unsigned deep, int mode)
+{
+    if (lower == 0) return false;  // nothing to go down to
+    const int k = int((e >> 3) & 7u);
+    bool ok = (e & kTabDestructible) != 0;
+    if (!ok && (e & kTabDivergent)) {
+        unsigned has_shallow = 0, has_deep = 0;  // by component
+        for (int i = 0; i < 8; ++i) {
+            const unsigned lab = (e >> (kTabLabelShift + 3 * i)) & 7u;
+            if (lab == 0) continue;
+            if ((deep >> i) & 1u) has_deep |= 1u << (lab - 1);
+            else has_shallow |= 1u << (lab - 1);
+        }
+        int fit = 0;
+        for (int j = 0; j < k; ++j) fit += (mode & 1) ? !((has_deep >> j) & 1u) : ((has_shallow >> j) & 1u);
+        ok = fit + 1 >= k;
+    }
+    if (mode & 2) {
+        const bool shallow = (lower & ~deep) != 0;  // F(x) - alpha^- <= lambda
+        const bool peak = (e & 7u) == 0;            // T+ = 0
+        const unsigned near = (mode & 4) ? 0x55u : 0xffu;  // Gamma_n^*(x): 4- or 8-neighbours
+        const unsigned up = ~lower & near;
+        const bool end = up != 0 && (up & (up - 1)) == 0;  // exactly one of them >= F(x)
+        ok = (ok || (peak && shallow)) && !(end && !shallow);
+    }
+    return ok;
+}
+
+constexpr DecisionTable make_decision_table()
+{
+    DecisionTable t{};
+    for (int i = 0; i < kDecisions; ++i) {
+        unsigned lower = 0, deep = 0;
+        for (int d = 0, r = i; d < 8; ++d, r /= 3) {
+            if (r % 3 > 0) lower |= 1u << d;
+            if (r % 3 > 1) deep |= 1u << d;
+        }
+        for (int mode = 0; mode < 8; ++mode)
+            if (decision((mode & 4 ? kPointTable48 : kPointTable).v[lower], lower, deep, mode)) t.v[i] |= uint8_t(1u << mode);
+    }
+    return t;
+}
+
+constexpr DecisionTable kDecisionTable = make_decision_table();
 
 #ifdef __CUDACC__
 

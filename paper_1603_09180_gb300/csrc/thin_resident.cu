@@ -25,11 +25,9 @@
 // and appends the groups it finds to one queue of the block; after a block
 // barrier the queue is split evenly over ceil(N / 32) warps (at most all 16),
 // so a front that crosses only part of the image still keeps the block's
-// schedulers busy, and a sparse phase runs on full lanes of a few warps.  A warp whose share is
-// larger than 32 groups tests them all first, packing those that lower (with
-// their test result) to the front of its share, then lowers them on full
-// lanes starting from that result; with fewer it tests and lowers in one
-// pass.  One more block barrier ends the phase.
+// schedulers busy, and a sparse phase runs on full lanes of a few warps.  Each
+// group is lowered as it is tested (thin_simd.cuh).  One more block barrier ends
+// the phase.
 //
 // Wide mode.  An image too large for one cluster is spread over all clusters
 // of one cooperative launch, a strip each.  Halo rows cross between clusters
@@ -41,6 +39,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "thin_common.cuh"
@@ -57,36 +56,13 @@ namespace {
 // registers a thread either way).
 constexpr int kResMaxWarps = 16;
 constexpr int kResStep = 8;  // phases between halo exchanges = halo rows held from each neighbour
-// A warp with more queued groups than this tests them all first and lowers
-// the ones that qualify on packed lanes; with fewer it lowers as it tests.
-// The lowering pass starts from the test pass's result (one byte per group),
-// and the common mode (lambda-thinning, F^- = max, (8,4)) has its own build
-// of the point test.  Since only neighbours whose test can change are
-// marked, most tested groups lower, and re-gathering them in a second pass
-// costs more than packing saves: the four-point SIMD path always lowers as it
-// tests (the 192-job u8 batch went from 21.8 to 19.8 ms against a threshold
-// of 32 groups).  The table path tests first, whatever the count.
-constexpr int kTwoPass = 1 << 30;
-constexpr bool kOkPass = true;
-constexpr bool kFix = true;
-// Which neighbours of a lowered point become dirty (marks8 / marks16): 0 all
-// eight; 1 those above the point's new value; 2 those also at most its old
-// value + lambda (the second bound only outside the wide mode, where it was
-// measured to cost more than it saves).  The skipped ones cannot change their
-// test result.
-#ifndef THIN_RES_MARK
-#define THIN_RES_MARK 2
-#endif
-constexpr int kMark = THIN_RES_MARK;
-
-__device__ const PointTable d_res_point_table = kPointTable;
-__device__ const PointTable d_res_point_table48 = kPointTable48;
+__device__ const DecisionTable d_res_decisions = kDecisionTable;
 
 // Shared-memory map of one block for a job.
-constexpr int kOffTabs = 0;      // point tables of (8,4) and (4,8), 2 KiB (the block up to 4 KiB is free)
-constexpr int kOffCtrl = 4096;   // control words
-constexpr int kOffBar = 4352;    // mbarrier of the row staging
-constexpr int kOffRows = 4480;   // image rows (16-byte aligned)
+constexpr int kOffTab = 0;       // decision table
+constexpr int kOffCtrl = 6656;   // control words
+constexpr int kOffBar = 6912;    // mbarrier of the row staging
+constexpr int kOffRows = 7040;   // image rows (16-byte aligned)
 constexpr int kResMaxCluster = 16;  // largest cluster (16 is a non-portable size, used where the device allows)
 // Steps (exchanges of halo rows) a job runs before it yields its cluster to a
 // waiting job, when a launch has more jobs than clusters: 1024 phases of
@@ -104,6 +80,7 @@ struct Ctrl {
     unsigned fail[2];        // wide launches, cluster leader: a block's grid-barrier wait failed (by step parity)
     int yield;               // cluster leader: the job pauses at this time slice's end
 };
+static_assert(kOffTab + kDecisionBytes <= kOffCtrl, "the decision table overlaps the control words");
 static_assert(sizeof(Ctrl) <= kOffBar - kOffCtrl, "control words overlap the mbarrier");
 
 __host__ __device__ inline size_t res_bits_off(int rows, int rp) { return (kOffRows + size_t(rows) * rp + 15) / 16 * 16; }
@@ -123,8 +100,7 @@ __host__ __device__ inline int res_warp_queue(int rows, int wpr, int nw)
 }
 __host__ __device__ inline size_t res_smem_bytes(int rows, int rp, int wpr, int nw)
 {
-    // per warp: 16-bit group codes, then one byte per group (its test result)
-    return res_queue_off(rows, rp, wpr) + size_t(3) * nw * res_warp_queue(rows, wpr, nw) + 16;
+    return res_queue_off(rows, rp, wpr) + size_t(2) * nw * res_warp_queue(rows, wpr, nw) + 16;  // 16-bit group codes
 }
 
 __device__ __forceinline__ unsigned long long res_gtimer()
@@ -250,15 +226,11 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
     const int C = int(cluster.num_blocks());
     const int rank = int(cluster.block_rank());
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t *tabs = reinterpret_cast<uint32_t *>(smem + kOffTabs);
     Ctrl *ctrl = reinterpret_cast<Ctrl *>(smem + kOffCtrl);
     const uint32_t bar = res_smem_u32(smem + kOffBar);
     uint8_t *rows_base = smem + kOffRows;
 
-    for (int i = tid; i < 256; i += blockDim.x) {
-        tabs[i] = d_res_point_table.v[i];
-        tabs[kTabOffset48 + i] = d_res_point_table48.v[i];
-    }
+    load_decisions(smem + kOffTab, d_res_decisions);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -285,9 +257,9 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
         }
         const ResJob J = P.jobs[job];
         constexpr int es = ES;
-        const int mode = P.rule | (J.adj << 2);      // F^- reading, operator, adjacency pair
-        const bool simd = J.adj == 0;                // (8,4): four points at once (bytes for u8, 16-bit lanes for u16)
-        const uint32_t *ptab = tabs + (J.adj ? kTabOffset48 : 0);
+        using T = typename std::conditional<ES == 1, uint8_t, uint16_t>::type;
+        // mode: F^- reading, operator, adjacency pair
+        const PointRule rule = point_rule(smem + kOffTab, P.rule | (J.adj << 2), J.lam, ES, !wide);
         const int R = J.rows, HR = J.hr, RP = J.rp, CW = J.cw, WPR = J.wpr;
         const int LR = R + 2 * HR;   // shared rows: HR halo rows, R own rows, HR halo rows
         const int CRT = LR / 2;      // cell rows held
@@ -296,10 +268,8 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
         // dirty[q]: per parity q = 2 (y & 1) + (x & 1), one bit per 4-point group (cell row, column):
         // some neighbour of a point of the group moved since the group's last test
         uint32_t *dirty = reinterpret_cast<uint32_t *>(smem + res_bits_off(LR, RP));
-        // the block's queue of the groups found in one scan round (codes, then one test-result byte each)
-        const int WQ = res_warp_queue(LR, WPR, NW);
+        // the block's queue of the groups found in one scan round
         uint16_t *bqueue = reinterpret_cast<uint16_t *>(smem + res_queue_off(LR, RP, WPR));
-        uint8_t *bok = smem + res_queue_off(LR, RP, WPR) + size_t(2) * NW * WQ;
         const int row0 = gb * R;         // first own image row
         const int ybase = row0 - HR;     // image row of shared row 0
         const int rowb = J.w * es;
@@ -426,46 +396,12 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
                     cr = CW > 1 ? int(__umulhi(uint32_t(code), Mcw)) : code;
                     cc = code - cr * CW;
                     const int y = ybase + 2 * cr + py;
-                    vm = 0;
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        const int x = 8 * cc + px + 2 * kk;
-                        vm |= (x >= 1 && x <= J.w - 2 ? 1u : 0u) << (8 * kk);
-                    }
+                    const int last = (J.w - 2 - px - 8 * cc) >> 1;  // last point inside the image border
+                    vm = last >= 3 ? kLsb8 : last >= 0 ? kLsb8 >> (8 * (3 - last)) : 0u;
+                    if (px == 0 && cc == 0) vm &= ~1u;  // x = 0
                     in = (y >= row0 && y < row0 + R) ? vm : 0u;  // own points count
                 };
                 bool moved_own = false;
-                // the (8,4) point test on four points at once, in the common mode's own build where it applies
-                auto test_item = [&](const uint8_t *rb, int pxx, uint32_t vm) -> uint32_t {
-                    if constexpr (ES == 1) {
-                        return (kFix && mode == 0) ? test_u8<0>(rb - RP, rb, rb + RP, pxx, vm, J.lam, mode)
-                                                   : test_u8(rb - RP, rb, rb + RP, pxx, vm, J.lam, mode);
-                    } else {
-                        const uint16_t *r16 = reinterpret_cast<const uint16_t *>(rb);
-                        const int rp16 = RP / 2;
-                        return (kFix && mode == 0) ? test_u16<0>(r16 - rp16, r16, r16 + rp16, pxx, vm, J.lam, mode)
-                                                   : test_u16(r16 - rp16, r16, r16 + rp16, pxx, vm, J.lam, mode);
-                    }
-                };
-                // the lowering loop on four points (ok: a first test's result, or ~0u to test first);
-                // aff receives the neighbours to mark
-                auto lower_item = [&](uint8_t *rb, int pxx, uint32_t vm, uint32_t in, uint32_t ok, uint32_t &aff) -> uint32_t {
-                    if constexpr (ES == 1) {
-                        if (ok == ~0u)
-                            return (kFix && mode == 0)
-                                       ? item_u8<0, kMark>(rb - RP, rb, rb + RP, pxx, vm, in, J.lam, mode, nlow, aff, !wide)
-                                       : item_u8<-1, kMark>(rb - RP, rb, rb + RP, pxx, vm, in, J.lam, mode, nlow, aff, !wide);
-                        return (kFix && mode == 0)
-                                   ? item_u8_tested<0, kMark>(rb - RP, rb, rb + RP, pxx, vm, in, ok, J.lam, mode, nlow, aff, !wide)
-                                   : item_u8_tested<-1, kMark>(rb - RP, rb, rb + RP, pxx, vm, in, ok, J.lam, mode, nlow, aff, !wide);
-                    } else {
-                        uint16_t *r16 = reinterpret_cast<uint16_t *>(rb);
-                        const int rp16 = RP / 2;
-                        return (kFix && mode == 0)
-                                   ? item_u16<0, kMark>(r16 - rp16, r16, r16 + rp16, pxx, vm, in, ok, J.lam, mode, nlow, aff, !wide)
-                                   : item_u16<-1, kMark>(r16 - rp16, r16, r16 + rp16, pxx, vm, in, ok, J.lam, mode, nlow, aff, !wide);
-                    }
-                };
                 // A scan round: warp w takes the round's bitmap words 32 w .. 32 w + 31 of this parity
                 // (one per lane; a small bitmap keeps only the first warps scanning), consumes their bits
                 // and appends the groups it found to the block's queue.  After a block barrier the queue
@@ -516,76 +452,22 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
                     const int act = min(NW, (N + 31) >> 5);
                     const int qa = warp < act ? (N * warp) / act : N;
                     const int nq = warp < act ? (N * (warp + 1)) / act - qa : 0;  // queue slots qa .. qa + nq - 1
-                    uint16_t *wqueue = bqueue + qa;
-                    uint8_t *wok = bok + qa;
-                    if (nq > 0) {
-                        int nl = nq;
-                        if (!simd || nq > kTwoPass) {
-                            // test first; the groups that lower are packed to the front of the share
-                            // (in place: a chunk's slots are read before any of them is written)
-                            nl = 0;
-                            for (int kb = 0; kb < nq; kb += 32) {
-                                const int k = kb + lane;
-                                bool lowers = false;
-                                int code = 0, gcr = 0, gcc = 0;
-                                uint32_t tmoved = 0;
-                                if (k < nq) {
-                                    code = wqueue[k];
-                                    uint32_t vm, in;
-                                    where(code, gcr, gcc, vm, in);
-                                    ntest += __popc(in);
-                                    uint8_t *rb = rows_base + size_t(2 * gcr + py) * RP + 16 + size_t(8 * es) * gcc;
-                                    if (simd) {
-                                        const uint32_t okb = test_item(rb, px, vm);
-                                        lowers = okb != 0;
-                                        code |= int((okb | (okb >> 7) | (okb >> 14) | (okb >> 21)) & 0xfu) << 16;
-                                    } else {
-                                        if constexpr (ES == 2)
-                                            tmoved = item_table<uint16_t>(reinterpret_cast<const uint16_t *>(rb - RP),
-                                                                          reinterpret_cast<uint16_t *>(rb),
-                                                                          reinterpret_cast<const uint16_t *>(rb + RP), px,
-                                                                          vm, in, ptab, J.lam, mode, nlow);
-                                        else
-                                            tmoved = item_table<uint8_t>(rb - RP, rb, rb + RP, px, vm, in, ptab, J.lam,
-                                                                         mode, nlow);
-                                        if (tmoved & in) moved_own = true;
-                                    }
-                                }
-                                if (!simd) mark(gcr, gcc, tmoved * 0xffu);  // the table path marks every neighbour
-                                const unsigned bal = __ballot_sync(0xffffffffu, lowers);
-                                if (lowers) {
-                                    const int at = nl + __popc(bal & ((1u << lane) - 1u));
-                                    wqueue[at] = uint16_t(code);
-                                    wok[at] = uint8_t(code >> 16);  // which of the four points passed the test
-                                }
-                                nl += __popc(bal);
-                            }
-                            __syncwarp();
-                            if (!simd) nl = 0;
+                    const uint16_t *wqueue = bqueue + qa;
+                    for (int kb = 0; kb < nq; kb += 32) {
+                        const int k = kb + lane;
+                        int gcr = 0, gcc = 0;
+                        uint32_t aff = 0;
+                        if (k < nq) {
+                            const int code = wqueue[k];
+                            uint32_t vm, in;
+                            where(code, gcr, gcc, vm, in);
+                            ntest += int((in * kLsb8) >> 24);
+                            T *rb = reinterpret_cast<T *>(rows_base + size_t(2 * gcr + py) * RP + 16) + 8 * gcc;
+                            const T *ra = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) - RP);
+                            const T *rc = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) + RP);
+                            if (lower_item<true>(ra, rb, rc, px, vm, in, rule, nlow, aff) & in) moved_own = true;
                         }
-                        // lower them (u8, (8,4)); with few groups the loop's first test is the only one
-                        for (int kb = 0; kb < nl; kb += 32) {
-                            const int k = kb + lane;
-                            int gcr = 0, gcc = 0;
-                            uint32_t moved = 0, aff = 0;
-                            if (k < nl) {
-                                const int code = wqueue[k];
-                                uint32_t vm, in;
-                                where(code, gcr, gcc, vm, in);
-                                if (nq <= kTwoPass) ntest += __popc(in);
-                                uint8_t *rb = rows_base + size_t(2 * gcr + py) * RP + 16 + size_t(8 * es) * gcc;
-                                if (kOkPass && nq > kTwoPass) {  // tested in the first pass: start lowering at once
-                                    const uint32_t o4 = wok[k];
-                                    const uint32_t okb = (o4 & 1u) | ((o4 & 2u) << 7) | ((o4 & 4u) << 14) | ((o4 & 8u) << 21);
-                                    moved = lower_item(rb, px, vm, in, okb, aff);
-                                } else {
-                                    moved = lower_item(rb, px, vm, in, ~0u, aff);
-                                }
-                                if (moved & in) moved_own = true;
-                            }
-                            mark(gcr, gcc, aff);
-                        }
-                        __syncwarp();
+                        mark(gcr, gcc, aff);
                     }
                     if (r0 + 32 * NW < slot_words) __syncthreads();  // the next round refills the queue
                 }

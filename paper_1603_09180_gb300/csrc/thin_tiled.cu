@@ -48,7 +48,6 @@ namespace {
 constexpr int kWarps = 8;
 constexpr int kThreads = 32 * kWarps;
 constexpr int kMinHalo = 3;
-constexpr int kNever = -(1 << 30);  // stamp of a cell that never changes
 
 struct ImgDesc {
     CUtensorMap map[2];          // TMA descriptors of buffer 0 and buffer 1
@@ -108,8 +107,7 @@ struct EngineArgs {
     int debug;         // 1: block 0 never arrives at the first barrier (timeout test)
 };
 
-__device__ const PointTable d_point_table = kPointTable;
-__device__ const PointTable d_point_table48 = kPointTable48;
+__device__ const DecisionTable d_decisions = kDecisionTable;
 
 __device__ __forceinline__ unsigned long long gtimer()
 {
@@ -248,14 +246,14 @@ struct Visit {
 // the points of its parity within distance Hs-1-j of the tile and off the
 // image border; after Hs phases the tile interior is exact.
 template <typename T>
-__device__ void visit_phases(T *tile, int bw, int32_t *cells, int ccols, uint16_t *queue, const Visit &V,
-                             const uint32_t *tabs, int &nlow, int &chg_j, int &ntest)
+__device__ void visit_phases(T *tile, int bw, uint8_t *cells, int ccols, uint16_t *queue, const Visit &V,
+                             const uint8_t *tab, int &nlow, int &chg_j, int &ntest)
 {
+    const PointRule rule = point_rule(tab, V.rule, V.lam, sizeof(T), false);
     const int lane = threadIdx.x & 31;
     const unsigned lt_lanes = (1u << lane) - 1u;
     for (int j = 0; j < V.Hs; ++j) {
         const long long g = V.g0 + j;
-        const int rel = int(g - V.start);
         const int p = int(g & 3);
         const int px = p & 1, py = p >> 1;
         const int r = V.Hs - 1 - j;
@@ -279,11 +277,11 @@ __device__ void visit_phases(T *tile, int bw, int32_t *cells, int ccols, uint16_
                 const int rk = div_small(it, nq, Mq);
                 const int q = qlo + it - rk * nq;
                 const int sr = sra + 2 * rk;
-                const int32_t *cp = cells + ((sr >> 1) + 1) * ccols + q + 1;
-                int m = max(max(cp[-ccols - 1], cp[-ccols]), cp[-ccols + 1]);
-                m = max(m, max(max(cp[-1], cp[0]), cp[1]));
-                m = max(m, max(max(cp[ccols - 1], cp[ccols]), cp[ccols + 1]));
-                dirty = m >= rel - 3;
+                const uint8_t *cp = cells + ((sr >> 1) + 1) * ccols + q + 1;
+                uint32_t m = max(max(uint32_t(cp[-ccols - 1]), uint32_t(cp[-ccols])), uint32_t(cp[-ccols + 1]));
+                m = max(m, max(max(uint32_t(cp[-1]), uint32_t(cp[0])), uint32_t(cp[1])));
+                m = max(m, max(max(uint32_t(cp[ccols - 1]), uint32_t(cp[ccols])), uint32_t(cp[ccols + 1])));
+                dirty = m > uint32_t(j);  // a stamp of phase g - 3 or later
                 code = (sr << 6) | q;
             }
             const unsigned bal = __ballot_sync(0xffffffffu, dirty);
@@ -303,21 +301,11 @@ __device__ void visit_phases(T *tile, int bw, int32_t *cells, int ccols, uint16_
             const bool inside = unsigned(sr - V.hr) < unsigned(V.th) && sb >= V.pad && sb < V.pad + V.tw;
             const uint32_t in = inside ? vm : 0u;
             ntest += __popc(in);
-            uint32_t moved, aff;  // (this engine marks whole cells: aff is not used)
+            uint32_t aff;  // (this engine marks whole cells: aff is not used)
             T *rb = tile + sr * bw + sb;
-            if (sizeof(T) == 1 && !(V.rule & 4))  // u8 under (8,4): four points at once
-                moved = item_u8(reinterpret_cast<const uint8_t *>(rb - bw), reinterpret_cast<uint8_t *>(rb),
-                                reinterpret_cast<const uint8_t *>(rb + bw), px, vm, in, V.lam, V.rule,
-                                nlow, aff);
-            else if (sizeof(T) == 2 && !(V.rule & 4))  // u16 under (8,4): four points in 16-bit lanes
-                moved = item_u16(reinterpret_cast<const uint16_t *>(rb - bw), reinterpret_cast<uint16_t *>(rb),
-                                 reinterpret_cast<const uint16_t *>(rb + bw), px, vm, in, ~0u, V.lam,
-                                 V.rule, nlow, aff);
-            else
-                moved = item_table<T>(rb - bw, rb, rb + bw, px, vm, in, tabs + ((V.rule & 4) ? kTabOffset48 : 0), V.lam,
-                                      V.rule, nlow);
+            const uint32_t moved = lower_item<false>(rb - bw, rb, rb + bw, px, vm, in, rule, nlow, aff);
             if (moved) {
-                cells[((sr >> 1) + 1) * ccols + q + 1] = rel;
+                cells[((sr >> 1) + 1) * ccols + q + 1] = uint8_t(j + 4);
                 if (moved & in) chg = true;
             }
         }
@@ -362,27 +350,24 @@ __device__ __forceinline__ void decode(const EngineArgs &P, bool full, const uns
     tx = local - ty * D.tiles_x;
 }
 
-constexpr int kSmemTabs = 4 * kTabWords;  // point tables of (8,4) and (4,8), 256 x u32 each
+constexpr int kSmemTabs = (kDecisionBytes + 127) / 128 * 128;  // the decision table
 
 __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
 {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     // TMA destinations want 128-byte aligned shared addresses
     uint8_t *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    uint32_t *tabs = reinterpret_cast<uint32_t *>(smem);
+    const uint8_t *tabs = smem;
     __shared__ int s_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const WarpLayout WL = P.wl;
     uint8_t *wbase = smem + kSmemTabs + warp * WL.bytes;
     uint8_t *tile = wbase;
-    int32_t *cells = reinterpret_cast<int32_t *>(wbase + WL.cell_off);
+    uint8_t *cells = wbase + WL.cell_off;
     uint16_t *queue = reinterpret_cast<uint16_t *>(wbase + WL.queue_off);
     const uint32_t bar = smem_u32(wbase + WL.bar_off);
 
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-        tabs[i] = d_point_table.v[i];
-        tabs[kTabOffset48 + i] = d_point_table48.v[i];
-    }
+    load_decisions(smem, d_decisions);
     if (lane == 0) {
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -441,7 +426,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
                 const uint32_t bytes = uint32_t(bw * es * (P.th + 2 * HR));
                 tma_load_2d(smem_u32(tile), &D.map[src], V.x0 - V.pad, V.y0 - HR, bar, bytes);
             }
-            // stamps of the region (overlaps the load); the border ring never changes
+            // Stamps of the region (overlaps the load); the border ring never changes.  In shared
+            // memory a stamp is a byte, its distance from stamp0: 0 for anything before the last three
+            // phases (no phase of this step looks further back), 4 + j for phase j of the step.
+            const int stamp0 = int(g0 - P.start_phase) - 4;
             {
                 const int32_t *gc = reinterpret_cast<const int32_t *>(D.cells);
                 const int cx0 = (V.x0 - V.pad) / 8 - 1, cy0 = (V.y0 - HR) / 2 - 1;
@@ -451,9 +439,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
                     const int cy = div_small(e, WL.ccols, Mcc), cx = e - cy * WL.ccols;
                     const int gx = cx0 + cx, gy = cy0 + cy;
                     const bool ring = cx == 0 || cy == 0 || cx == WL.ccols - 1 || cy == WL.crows - 1;
-                    cells[e] = (!ring && gx >= 0 && gy >= 0 && gx < D.cells_x && gy < D.cells_y)
-                                   ? __ldcg(gc + size_t(gy) * D.cells_x + gx)
-                                   : kNever;
+                    int age = 0;
+                    if (!ring && gx >= 0 && gy >= 0 && gx < D.cells_x && gy < D.cells_y)
+                        age = max(__ldcg(gc + size_t(gy) * D.cells_x + gx) - stamp0, 0);
+                    cells[e] = uint8_t(age);
                 }
             }
             const bool ok = mbar_wait(bar, parity, P.timeout_ns);
@@ -486,7 +475,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
                     const int cy = div_small(e, icx, Mi), cx = e - cy * icx;
                     const int gx = cxa + cx, gy = cya + cy;
                     if (gx < D.cells_x && gy < D.cells_y)
-                        __stcg(gc + size_t(gy) * D.cells_x + gx, cells[(oy + cy) * WL.ccols + ox + cx]);
+                        __stcg(gc + size_t(gy) * D.cells_x + gx, stamp0 + cells[(oy + cy) * WL.ccols + ox + cx]);
                 }
             }
             nlow = __reduce_add_sync(0xffffffffu, nlow);
@@ -592,7 +581,7 @@ WarpLayout warp_layout(int tw, int th, int hr, bool any16)
     L.crows = rows / 2 + 2;
     L.cell_off = L.tile_bytes;
     const int max_items = (rows / 2 + 1) * (cols8 + 1);
-    L.queue_off = int(align_up(size_t(L.cell_off) + 4 * size_t(L.ccols) * L.crows, 16));
+    L.queue_off = int(align_up(size_t(L.cell_off) + size_t(L.ccols) * L.crows, 16));
     L.bar_off = int(align_up(size_t(L.queue_off) + 2 * size_t(max_items), 16));
     L.bytes = int(align_up(size_t(L.bar_off) + 16, 128));
     return L;
