@@ -72,19 +72,18 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     G->resident.clear();
     G->wide.clear();
     G->tiled.clear();
-    G->nw = 16;  // warps per resident block (one block per SM measured fastest)
     std::vector<int> cls(n, 0);
     if (o.kernel == THIN_KERNEL_AUTO || o.kernel == THIN_KERNEL_RESIDENT) {
-        const size_t limit = resident_smem_limit(16 / G->nw);
+        const size_t limit = resident_smem_limit();
         for (int k = 0; k < n; ++k)
-            cls[k] = resident_cluster_size(specs[k].w, specs[k].h, specs[k].dtype, limit, G->nw, nullptr, nullptr);
+            cls[k] = resident_cluster_size(specs[k].w, specs[k].h, specs[k].dtype, limit, nullptr, nullptr);
     }
     int eligible = 0, sms = 0, dev = 0;
     for (int k = 0; k < n; ++k) eligible += cls[k] > 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int spread = 1;
-    while (eligible > 0 && spread < 8 && spread * 2 * eligible <= sms * (16 / G->nw)) spread *= 2;
+    while (eligible > 0 && spread < 8 && spread * 2 * eligible <= sms) spread *= 2;
     // one launch per cluster size and element size (the kernel is built for each element size)
     for (int C = 1; C <= 16; C *= 2)
         for (int dt = THIN_U8; dt <= THIN_U16; ++dt) {
@@ -102,10 +101,10 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     // the call, each then having most of the GPU; the tiled engine otherwise.
     std::vector<int> strips(n, 0), csize(n, 0);
     if (allow_wide && (o.kernel == THIN_KERNEL_AUTO || o.kernel == THIN_KERNEL_RESIDENT)) {
-        const size_t limit = resident_smem_limit(16 / G->nw);
+        const size_t limit = resident_smem_limit();
         for (int k = 0; k < n; ++k)
             if (cls[k] == 0)
-                strips[k] = resident_wide_strips(specs[k].w, specs[k].h, specs[k].dtype, limit, G->nw, &csize[k]);
+                strips[k] = resident_wide_strips(specs[k].w, specs[k].h, specs[k].dtype, limit, &csize[k]);
     }
     int nwide = 0;
     for (int k = 0; k < n; ++k) nwide += cls[k] == 0 && strips[k] > 0;
@@ -173,13 +172,13 @@ int Execution::prepare(const std::vector<JobSpec> &specs_in, const Grouping &G, 
         res.emplace_back();
         res_idx.push_back(grp.second);
         const int rc =
-            resident_prepare(js.data(), int(js.size()), grp.first, G.nw, o, s, async_alloc, &res.back(), 0, done);
+            resident_prepare(js.data(), int(js.size()), grp.first, o, s, async_alloc, &res.back(), 0, done);
         if (rc != THIN_OK) return rc;
     }
     for (const auto &wj : G.wide) {
         wide.emplace_back();
         wide_idx.push_back(wj.job);
-        const int rc = resident_prepare(&specs[wj.job], 1, wj.C, G.nw, o, s, async_alloc, &wide.back(), wj.strips);
+        const int rc = resident_prepare(&specs[wj.job], 1, wj.C, o, s, async_alloc, &wide.back(), wj.strips);
         if (rc != THIN_OK) return rc;
     }
     if (!G.tiled.empty()) {

@@ -135,7 +135,7 @@ struct ResArgs {
 // be enqueued any number of times: see resident_prepare / _enqueue /
 // _collect / _release.
 struct ResidentPrepared {
-    int n = 0, C = 0, nw = 0, grid = 0, strips = 0, es = 1;
+    int n = 0, C = 0, grid = 0, strips = 0, es = 1;
     size_t smem = 0;
     bool async_alloc = true;
     char *base = nullptr;         // one device allocation holding everything below
@@ -146,24 +146,24 @@ struct ResidentPrepared {
 };
 // strips > 0: one image (n == 1) over `strips` clusters of C blocks, one
 // cooperative launch (the wide mode for images larger than one cluster).
-int resident_prepare(const JobSpec *jobs, int n, int C, int nw, const thin_options &opt, cudaStream_t stream,
+int resident_prepare(const JobSpec *jobs, int n, int C, const thin_options &opt, cudaStream_t stream,
                      bool async_alloc, ResidentPrepared *R, int strips = 0, ResDone *done = nullptr);
 cudaError_t resident_enqueue(const ResidentPrepared &R, cudaStream_t stream);
 int resident_collect(const ResidentPrepared &R, const thin_options &opt, cudaStream_t stream, thin_stats *out);
 // The public stats of a finished resident job (error: the launch's error word).
 void resident_stats(const ResStat &S, int error, const thin_options &opt, thin_stats *o);
 void resident_release(ResidentPrepared &R, cudaStream_t stream);
-// Smallest cluster of nw-warp blocks whose shared memory holds a w x h image
+// Smallest cluster whose shared memory holds a w x h image
 // of `dtype`, 0 if none.
-int resident_cluster_size(int w, int h, int dtype, size_t smem_limit, int nw, int *rows_out, int *rp_out);
+int resident_cluster_size(int w, int h, int dtype, size_t smem_limit, int *rows_out, int *rp_out);
 // Largest resident cluster on the current device: 16 where it can run, else 8.
-int resident_max_cluster(int nw, size_t smem_limit);
-// Shared memory one block may take when `blocks` blocks share an SM.
-size_t resident_smem_limit(int blocks);
-// Wide mode: the fewest strips (clusters of *c_out blocks of nw warps, the
+int resident_max_cluster(size_t smem_limit);
+// Shared memory one block may take (one block per SM).
+size_t resident_smem_limit();
+// Wide mode: the fewest strips (clusters of *c_out blocks, the
 // largest cluster size that works) whose shared memory holds the image, all
 // clusters resident at once; 0 if none.
-int resident_wide_strips(int w, int h, int dtype, size_t smem_limit, int nw, int *c_out);
+int resident_wide_strips(int w, int h, int dtype, size_t smem_limit, int *c_out);
 
 // A tiled launch prepared on the host (opaque; thin_tiled.cu).
 struct TiledPrepared;
@@ -188,7 +188,6 @@ constexpr int kMaxResidentGroups = 10;
 // Launch groups of a batch: (cluster size, job indices) for the resident
 // engine, job indices for the tiled engine.
 struct Grouping {
-    int nw = 16;
     std::vector<std::pair<int, std::vector<int>>> resident;
     struct Wide {
         int job, strips, C;

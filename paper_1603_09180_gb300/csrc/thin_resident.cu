@@ -21,13 +21,22 @@
 // changed nothing anywhere in the image (its fixed point under the schedule)
 // or at the phase cap.
 //
-// Work in a phase.  Each warp scans its share of the parity's bitmap words
-// and appends the groups it finds to one queue of the block; after a block
-// barrier the queue is split evenly over ceil(N / 32) warps (at most all 16),
-// so a front that crosses only part of the image still keeps the block's
-// schedulers busy, and a sparse phase runs on full lanes of a few warps.  Each
-// group is lowered as it is tested (thin_simd.cuh).  One more block barrier ends
-// the phase.
+// Work in a phase.  Each thread looks at one piece of the parity's bitmap and
+// appends the groups it finds to one queue of the block; after a block barrier
+// the queue goes to the warps in chunks of 32 groups, in turn, so a front that
+// crosses only part of the image still keeps the block's schedulers busy.  Each
+// group is lowered as it is tested (thin_simd.cuh), one thread to its four
+// points, or a lane to each point in a phase with few groups.  One more block
+// barrier ends the phase.
+//
+// What bounds it.  Busy phases (hundreds of groups a block) are bound by issue:
+// 1.9 to 2.1 warp instructions a cycle and SM, the FMA pipe 43 % and the ALU
+// pipe 32 % busy.  Sparse ones are a chain of latencies: scan, queue, gather,
+// two to four tests, marks, two block barriers, about 3000 cycles.
+// 192 512^2 images: 16.4 -> 14.5 ms (u8), 27.7 -> 23.2 ms (u16); 64^2 alone
+// 319 -> 264 us; 4096^2 u8 at lambda = 30 48.5 -> 42.5 ms (each against one
+// 32-bit word a lane in the scan, even shares of the queue for all warps and
+// divisions to find a group's cell).
 //
 // Wide mode.  An image too large for one cluster is spread over all clusters
 // of one cooperative launch, a strip each.  Halo rows cross between clusters
@@ -52,9 +61,14 @@ namespace thin {
 
 namespace {
 
-// Warps per block: 16, 8 or 4, with 1, 2 or 4 blocks per SM (at most 128
-// registers a thread either way).
-constexpr int kResMaxWarps = 16;
+// Warps per block, one block per SM (at most 128 registers a thread).
+constexpr int kResWarps = 16;
+constexpr int kResThreads = 32 * kResWarps;
+// Phases with at most this many groups in a block take a lane to a point (four
+// to a group): 64^2 at lambda = 10 245 -> 220 us, 192 512^2 u16 images
+// 24.1 -> 23.9 ms; at 256 a block's lanes take two turns, and the u8 batch lost
+// 3 %.
+constexpr int kLaneItems = 128;
 constexpr int kResStep = 8;  // phases between halo exchanges = halo rows held from each neighbour
 __device__ const DecisionTable d_res_decisions = kDecisionTable;
 
@@ -89,18 +103,24 @@ __host__ __device__ inline size_t res_queue_off(int rows, int rp, int wpr)
 {
     return res_bits_off(rows, rp) + size_t(4) * 4 * (rows / 2) * wpr;
 }
-// A scan round covers min(words, 32 nw) bitmap words of 32 groups each, and
-// the block's queue holds every group one round can find: nw x this many
-// entries (32 groups per word times min(ceil(words / nw), 32) words).
-__host__ __device__ inline int res_warp_queue(int rows, int wpr, int nw)
+// A scan round covers this many bitmap words (32 groups each); the block's
+// queue holds every group that one round can find, as 16-bit codes.  A small
+// bitmap is looked at in pieces of 8 or 16 bits, so that more threads share its
+// groups.
+constexpr int kScanWords = kResThreads;
+__host__ __device__ inline size_t res_smem_bytes(int rows, int rp, int wpr)
 {
     const int words = (rows / 2) * wpr;
-    const int per_warp = (words + nw - 1) / nw;
-    return (per_warp < 32 ? per_warp : 32) * 32;
+    return res_queue_off(rows, rp, wpr) + size_t(2) * 32 * (words < kScanWords ? words : kScanWords) + 16;
 }
-__host__ __device__ inline size_t res_smem_bytes(int rows, int rp, int wpr, int nw)
+
+// Group codes are 16-bit: cell row << ceil(log2(cells a row)) | cell column.
+// (The shared memory ends first: a cell holds 16 pixels.)
+inline bool codes_fit(int held, int cw)
 {
-    return res_queue_off(rows, rp, wpr) + size_t(2) * nw * res_warp_queue(rows, wpr, nw) + 16;  // 16-bit group codes
+    int bits = 0;
+    while ((1 << bits) < cw) ++bits;
+    return (size_t(held / 2) << bits) <= 65536;
 }
 
 __device__ __forceinline__ unsigned long long res_gtimer()
@@ -209,17 +229,15 @@ __device__ void res_push(const ResArgs &P, int job)
     *reinterpret_cast<volatile unsigned *>(&P.tag[s]) = 1u + t / P.cap;
 }
 
-// OR of m into bits[key] (key < 0: nothing to mark).  Combining the lanes
-// that name the same word first (__match_any_sync + __reduce_or_sync) was
-// measured slower than letting the shared-memory atomics serialise.
-__device__ __forceinline__ void or_word(uint32_t *bits, int key, uint32_t m)
+// ORs m into a word of shared memory; nothing where m is 0 (a predicate, not a branch).
+__device__ __forceinline__ void smem_or(uint32_t addr, uint32_t m)
 {
-    if (key >= 0) atomicOr(bits + key, m);
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %1, 0;\n @p red.shared.or.b32 [%0], %1;\n}\n" ::"r"(addr), "r"(m) : "memory");
 }
 
 // ES: element size of every image of the launch (1: u8, 2: u16).
-template <int NW, int ES>
-__global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs P)
+template <int ES>
+__global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs P)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     cg::cluster_group cluster = cg::this_cluster();
@@ -265,11 +283,13 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
         const int CRT = LR / 2;      // cell rows held
         const int HC = HR / 2;       // halo cell rows on each side
         const int slot_words = CRT * WPR;
+        const int unit = slot_words * 4 <= kResThreads ? 0 : slot_words * 2 <= kResThreads ? 1 : 2;  // scan pieces: 8 << unit bits
         // dirty[q]: per parity q = 2 (y & 1) + (x & 1), one bit per 4-point group (cell row, column):
         // some neighbour of a point of the group moved since the group's last test
         uint32_t *dirty = reinterpret_cast<uint32_t *>(smem + res_bits_off(LR, RP));
         // the block's queue of the groups found in one scan round
         uint16_t *bqueue = reinterpret_cast<uint16_t *>(smem + res_queue_off(LR, RP, WPR));
+        const uint32_t dirty_s = res_smem_u32(dirty);
         const int row0 = gb * R;         // first own image row
         const int ybase = row0 - HR;     // image row of shared row 0
         const int rowb = J.w * es;
@@ -337,8 +357,25 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
         // decisions and their cluster barriers stop pairing.
         cluster.sync();
 
+        // A group's code is (cell row << cbits) | cell column.
+        const int cbits = 32 - __clz(CW - 1);
+        // This thread's piece of a bitmap: the word, where its bits lie, the columns that exist, the
+        // code of its first group.  It stays the same for the whole job unless the bitmap needs several
+        // scan rounds.
+        int pword = 0, pshift = 0, prow = 0, pcode = 0;
+        uint32_t pmask = 0;
         const uint32_t Mwpr = WPR > 1 ? 0xffffffffu / uint32_t(WPR) + 1u : 0u;
-        const uint32_t Mcw = CW > 1 ? 0xffffffffu / uint32_t(CW) + 1u : 0u;
+        auto take_piece = [&](int r0) {
+            const int u = (r0 << (2 - unit)) + tid;
+            pword = u >> (2 - unit);
+            pshift = (u << (3 + unit)) & 31;
+            prow = WPR > 1 ? int(__umulhi(uint32_t(pword), Mwpr)) : pword;
+            const int cc = (pword - prow * WPR) * 32 + pshift;
+            const int valid = min(CW - cc, 8 << unit);
+            pmask = pword >= slot_words || valid <= 0 ? 0u : valid >= 32 ? 0xffffffffu : (1u << valid) - 1u;
+            pcode = (prow << cbits) | cc;
+        };
+        take_piece(0);
 
         long long g = run.resumed ? run.g : P.start_phase;
         unsigned qround = 0;  // scan rounds so far: selects the queue counter
@@ -353,92 +390,69 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
             for (int j = 0; j < Hs; ++j, ++g) {
                 const int p = int(g & 3), px = p & 1, py = p >> 1;
                 uint32_t *dp = dirty + p * slot_words;
-                // rows whose points are exact in this phase: own rows and Hs-1-j halo rows
-                const int rr = B > 1 ? Hs - 1 - j : 0;
-                const int ylo = max(1, row0 - rr), yhi = min(J.h - 2, row0 + R - 1 + rr);
                 // the groups of the other three parities holding a neighbour to test again become
                 // dirty.  A: byte k holds the ring directions (bit 0 E, 1 NE, 2 N, 3 NW, 4 W, 5 SW,
                 // 6 S, 7 SE) of point k's neighbours to mark; 0: nothing to mark.  E and W neighbours
                 // are in the row's other column parity, N and S in the other row parity, the
                 // diagonals in the fourth.  For px == 0 the W side of point 0 is in the cell to the
                 // left; for px == 1 the E side of point 3 is in the cell to the right.
-                const int qrow = 2 * py + (px ^ 1), qcol = 2 * (py ^ 1) + px, qdiag = 2 * (py ^ 1) + (px ^ 1);
+                const uint32_t pbytes = 4u * uint32_t(slot_words), up = py ? 0u : 0u - 4u * uint32_t(WPR);
+                const uint32_t qrow = pbytes * uint32_t(2 * py + (px ^ 1)), qcol = pbytes * uint32_t(2 * (py ^ 1) + px) + up,
+                               qdiag = pbytes * uint32_t(2 * (py ^ 1) + (px ^ 1)) + up;
                 auto mark = [&](int cr, int cc, uint32_t A) {
-                    const uint32_t rs = A & (px ? 0x10111111u : 0x11111101u);  // same cell: E, W
-                    const uint32_t as = A & (px ? 0x080a0a0au : 0x0a0a0a02u);  // NE, NW
-                    const uint32_t bs = A & (px ? 0x20a0a0a0u : 0xa0a0a080u);  // SE, SW
-                    const uint32_t rx = A & (px ? 0x01000000u : 0x00000010u);  // the cell beside
-                    const uint32_t ax = A & (px ? 0x02000000u : 0x00000008u);
-                    const uint32_t bx = A & (px ? 0x80000000u : 0x00000020u);
-                    const int w = cc >> 5, b = cc & 31;
-                    const uint32_t mc = 1u << b;
-                    const bool edge = px ? b == 31 : b == 0;  // the cell beside is in the next word
-                    const uint32_t mx = edge ? 0u : (px ? mc << 1 : mc >> 1);
-                    const uint32_t mrow = (rs ? mc : 0u) | (rx ? mx : 0u);
-                    const uint32_t ma = (as ? mc : 0u) | (ax ? mx : 0u);
-                    const uint32_t mb = (bs ? mc : 0u) | (bx ? mx : 0u);
-                    const int ca = cr - 1 + py, cb = cr + py;  // cell rows of rows y - 1, y + 1
-                    const bool va = ca >= 0, vb = cb < CRT;
-                    or_word(dirty, mrow ? qrow * slot_words + cr * WPR + w : -1, mrow);
-                    or_word(dirty, va && (A & 0x04040404u) ? qcol * slot_words + ca * WPR + w : -1, mc);
-                    or_word(dirty, va && ma ? qdiag * slot_words + ca * WPR + w : -1, ma);
-                    or_word(dirty, vb && (A & 0x40404040u) ? qcol * slot_words + cb * WPR + w : -1, mc);
-                    or_word(dirty, vb && mb ? qdiag * slot_words + cb * WPR + w : -1, mb);
-                    if (edge && (rx | ax | bx)) {  // the group across a word boundary (rare)
-                        const int ws = px ? w + 1 : w - 1;
-                        const uint32_t ms = px ? 1u : 0x80000000u;
-                        if (rx) atomicOr(&dirty[qrow * slot_words + cr * WPR + ws], ms);
-                        if (va && ax) atomicOr(&dirty[qdiag * slot_words + ca * WPR + ws], ms);
-                        if (vb && bx) atomicOr(&dirty[qdiag * slot_words + cb * WPR + ws], ms);
+                    const uint32_t beside = px ? 0x83000000u : 0x00000038u;  // towards the cell beside
+                    const uint32_t X = A & beside, x = px ? X >> 24 : X;
+                    uint32_t f = A ^ X;  // the rest, folded into one set of directions
+                    f |= f >> 16;
+                    f |= f >> 8;
+                    const uint32_t mc = 1u << (cc & 31);
+                    const uint32_t mx = px ? mc << 1 : mc >> 1;  // 0: the cell beside is in the next word
+                    const uint32_t mrow = (f & 0x11u ? mc : 0u) | (x & 0x11u ? mx : 0u);
+                    const uint32_t ma = (f & 0x0au ? mc : 0u) | (x & 0x0au ? mx : 0u);
+                    const uint32_t mb = (f & 0xa0u ? mc : 0u) | (x & 0xa0u ? mx : 0u);
+                    // word of the group's own cell in the bitmap of each parity; of the cell row of y - 1
+                    const uint32_t o = dirty_s + 4u * uint32_t(cr * WPR + (cc >> 5));
+                    const uint32_t drow = o + qrow, dcol = o + qcol, ddiag = o + qdiag;
+                    const uint32_t below = 4u * uint32_t(WPR);
+                    smem_or(drow, mrow);
+                    smem_or(dcol, f & 0x04u ? mc : 0u);
+                    smem_or(ddiag, ma);
+                    smem_or(dcol + below, f & 0x40u ? mc : 0u);
+                    smem_or(ddiag + below, mb);
+                    if (mx == 0u && x) {  // the group across a word boundary (rare)
+                        const uint32_t ws = px ? 4u : ~3u, ms = px ? 1u : 0x80000000u;
+                        smem_or(drow + ws, x & 0x11u ? ms : 0u);
+                        smem_or(ddiag + ws, x & 0x0au ? ms : 0u);
+                        smem_or(ddiag + below + ws, x & 0xa0u ? ms : 0u);
                     }
                 };
-                auto where = [&](int code, int &cr, int &cc, uint32_t &vm, uint32_t &in) {
-                    cr = CW > 1 ? int(__umulhi(uint32_t(code), Mcw)) : code;
-                    cc = code - cr * CW;
-                    const int y = ybase + 2 * cr + py;
-                    const int last = (J.w - 2 - px - 8 * cc) >> 1;  // last point inside the image border
-                    vm = last >= 3 ? kLsb8 : last >= 0 ? kLsb8 >> (8 * (3 - last)) : 0u;
-                    if (px == 0 && cc == 0) vm &= ~1u;  // x = 0
-                    in = (y >= row0 && y < row0 + R) ? vm : 0u;  // own points count
-                };
                 bool moved_own = false;
-                // A scan round: warp w takes the round's bitmap words 32 w .. 32 w + 31 of this parity
-                // (one per lane; a small bitmap keeps only the first warps scanning), consumes their bits
-                // and appends the groups it found to the block's queue.  After a block barrier the queue
-                // is split over the warps, and each warp tests and lowers its share on its own: no other
-                // block barrier until the end of the phase (or of the round, when the bitmap needs several).
-                for (int r0 = 0; r0 < slot_words; r0 += 32 * NW) {
-                    {
-                        const int wi = r0 + warp * 32 + lane;  // 32 consecutive words a warp: few warps scan
-                        uint32_t d = 0;
-                        int cr = 0;
-                        if (wi < slot_words) {
-                            cr = WPR > 1 ? int(__umulhi(uint32_t(wi), Mwpr)) : wi;
-                            const int i = wi - cr * WPR;
-                            const int y = ybase + 2 * cr + py;
-                            if (y >= ylo && y <= yhi) {
-                                const int valid = CW - 32 * i;
-                                d = dp[wi] & (valid >= 32 ? 0xffffffffu : ((1u << valid) - 1u));
-                            }
-                            if (dp[wi]) dp[wi] = 0u;
-                        }
-                        const int cnt = __popc(d);
-                        int incl = cnt;
+                // A scan round: each thread takes one piece of the parity's bitmap (a byte, or 16 or
+                // 32 bits where there are more of them than threads), consumes its bits and appends the
+                // groups it found to the block's queue.  After a block barrier the queue is worked on in
+                // chunks: no other block barrier until the end of the phase (or of the round, when the
+                // bitmap needs several).
+                for (int r0 = 0; r0 < slot_words; r0 += kScanWords) {
+                    if (slot_words > kScanWords) take_piece(r0);
+                    if (pmask) {
+                        uint32_t d = (dp[pword] >> pshift) & pmask;
+                        if (d) {
+                            if (unit == 0) reinterpret_cast<uint8_t *>(dp)[pword * 4 + (pshift >> 3)] = 0;
+                            else if (unit == 1) reinterpret_cast<uint16_t *>(dp)[pword * 2 + (pshift >> 4)] = 0;
+                            else dp[pword] = 0;
+                            // rows whose points are exact in this phase: own rows and Hs-1-j halo rows, off the
+                            // image border (rows y - 1 and y + 1 of each are held)
+                            const int rr = B > 1 ? Hs - 1 - j : 0, y = ybase + 2 * prow + py;
+                            if (y >= max(1, row0 - rr) && y <= min(J.h - 2, row0 + R - 1 + rr)) {
+                                uint16_t *q = bqueue + atomicAdd(&ctrl->qn[qround & 1], unsigned(__popc(d)));
+                                int code = pcode;
+                                do {
 #pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                            if (lane >= o) incl += v;
-                        }
-                        const int wsum = __shfl_sync(0xffffffffu, incl, 31);
-                        if (wsum) {
-                            int base = 0;
-                            if (lane == 31) base = int(atomicAdd(&ctrl->qn[qround & 1], unsigned(wsum)));
-                            int pos = __shfl_sync(0xffffffffu, base, 31) + incl - cnt;
-                            const int cbase = (wi - cr * WPR) * 32 + cr * CW;
-                            while (d) {
-                                const int bb = __ffs(d) - 1;
-                                d &= d - 1;
-                                bqueue[pos++] = uint16_t(cbase + bb);
+                                    for (int b = 0; b < 8; ++b)
+                                        if ((d >> b) & 1u) *q++ = uint16_t(code + b);
+                                    code += 8;
+                                    d >>= 8;
+                                } while (d);
                             }
                         }
                     }
@@ -446,35 +460,51 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
                     const int N = int(*reinterpret_cast<volatile unsigned *>(&ctrl->qn[qround & 1]));
                     if (tid == 0) ctrl->qn[(qround + 1) & 1] = 0u;  // last read in the previous round
                     ++qround;
-                    // The shares go to as few warps as give every warp a full chunk of 32 (all 16 when
-                    // there are more than 512 groups): a sparse phase then issues its groups on full
-                    // lanes from about one warp per scheduler instead of a few lanes of every warp.
-                    const int act = min(NW, (N + 31) >> 5);
-                    const int qa = warp < act ? (N * warp) / act : N;
-                    const int nq = warp < act ? (N * (warp + 1)) / act - qa : 0;  // queue slots qa .. qa + nq - 1
-                    const uint16_t *wqueue = bqueue + qa;
-                    for (int kb = 0; kb < nq; kb += 32) {
-                        const int k = kb + lane;
-                        int gcr = 0, gcc = 0;
-                        uint32_t aff = 0;
-                        if (k < nq) {
-                            const int code = wqueue[k];
-                            uint32_t vm, in;
-                            where(code, gcr, gcc, vm, in);
+                    if (N <= kLaneItems) {
+                        // few groups: a lane to a point
+                        for (int k = tid >> 2; k < N; k += kResThreads / 4) {
+                            const int code = bqueue[k], j4 = lane & 3;
+                            const int cr = code >> cbits, cc = code - (cr << cbits);
+                            const int x = 8 * cc + px + 2 * j4;
+                            if (x >= 1 && x <= J.w - 2) {
+                                T *rb = reinterpret_cast<T *>(rows_base + (2 * cr + py) * RP + 16) + x;
+                                const T *ra = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) - RP);
+                                const T *rc = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) + RP);
+                                uint32_t A;
+                                const int n = lower_one<T>(ra, rb, rc, rule, A);
+                                if (unsigned(cr - HC) < unsigned(R / 2)) {  // own rows count
+                                    ++ntest;
+                                    nlow += n;
+                                    moved_own |= n > 0;
+                                }
+                                if (A) mark(cr, cc, A << (8 * j4));
+                            }
+                        }
+                    } else {
+                        // Chunks of 32 groups go to the warps in turn: every chunk but the last is full, and
+                        // the schedulers' shares differ by one chunk at most.
+                        for (int k = tid; k < N; k += kResThreads) {
+                            const int code = bqueue[k];
+                            const int cr = code >> cbits, cc = code - (cr << cbits);
+                            const int last = (J.w - 2 - px - 8 * cc) >> 1;  // last point inside the image border
+                            uint32_t vm = last >= 3 ? kLsb8 : last >= 0 ? kLsb8 >> (8 * (3 - last)) : 0u;
+                            if (px == 0 && cc == 0) vm &= ~1u;  // x = 0
+                            const uint32_t in = unsigned(cr - HC) < unsigned(R / 2) ? vm : 0u;  // own rows count
                             ntest += int((in * kLsb8) >> 24);
-                            T *rb = reinterpret_cast<T *>(rows_base + size_t(2 * gcr + py) * RP + 16) + 8 * gcc;
+                            T *rb = reinterpret_cast<T *>(rows_base + (2 * cr + py) * RP + 16) + 8 * cc;
                             const T *ra = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) - RP);
                             const T *rc = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) + RP);
-                            if (lower_item<true>(ra, rb, rc, px, vm, in, rule, nlow, aff) & in) moved_own = true;
+                            uint32_t aff;
+                            moved_own |= (lower_item<true>(ra, rb, rc, px, vm, in, rule, nlow, aff) & in) != 0;
+                            if (aff) mark(cr, cc, aff);
                         }
-                        mark(gcr, gcc, aff);
                     }
-                    if (r0 + 32 * NW < slot_words) __syncthreads();  // the next round refills the queue
+                    if (r0 + kScanWords < slot_words) __syncthreads();  // the next round refills the queue
                 }
-                if (__syncthreads_or(moved_own) && tid == 0) ctrl->last = g;
+                if (moved_own) ctrl->last = g;  // (every writer writes the same value)
+                __syncthreads();
             }
             // ---- end of a step: every block's last change, then the stop test
-            __syncthreads();
             const int sp = int(steps & 1);  // buffer of this step in the exchange snapshot
             ++steps;
             long long lc = -1;
@@ -675,14 +705,14 @@ __global__ void __launch_bounds__(NW * 32, kResMaxWarps / NW) k_resident(ResArgs
     }
 }
 
-// Launch shape of k_resident<NW, ES>: as many clusters of C blocks as fit at
+// Launch shape of k_resident<ES>: as many clusters of C blocks as fit at
 // once (each loops over the job queue), at most one per job.
-template <int NW, int ES>
+template <int ES>
 cudaError_t resident_shape(int C, int n, size_t smem, int *grid)
 {
-    cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void *>(k_resident<NW, ES>));
+    cudaError_t e = allow_max_dynamic_smem(reinterpret_cast<const void *>(k_resident<ES>));
     if (e == cudaSuccess && C > 8)
-        e = cudaFuncSetAttribute(reinterpret_cast<const void *>(k_resident<NW, ES>),
+        e = cudaFuncSetAttribute(reinterpret_cast<const void *>(k_resident<ES>),
                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof cfg);
@@ -691,13 +721,13 @@ cudaError_t resident_shape(int C, int n, size_t smem, int *grid)
     attr[0].val.clusterDim.x = C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(NW * 32);
+    cfg.blockDim = dim3(kResThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.gridDim = dim3(C);
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int clusters = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, k_resident<NW, ES>, &cfg);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, k_resident<ES>, &cfg);
     if (e == cudaSuccess && clusters < 1) e = cudaErrorInvalidConfiguration;
     *grid = C * std::min(clusters, n);
     return e;
@@ -705,7 +735,7 @@ cudaError_t resident_shape(int C, int n, size_t smem, int *grid)
 
 // Wide launches are cooperative: the clusters of one image wait on one
 // another at every step, so all of them must be resident at once.
-template <int NW, int ES>
+template <int ES>
 cudaError_t resident_launch(int C, int grid, size_t smem, cudaStream_t stream, const ResArgs &P)
 {
     cudaLaunchConfig_t cfg;
@@ -717,28 +747,27 @@ cudaError_t resident_launch(int C, int grid, size_t smem, cudaStream_t stream, c
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeCooperative;
     attr[1].val.cooperative = 1;
-    cfg.blockDim = dim3(NW * 32);
+    cfg.blockDim = dim3(kResThreads);
     cfg.gridDim = dim3(grid);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = P.strips > 0 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, k_resident<NW, ES>, P);
+    return cudaLaunchKernelEx(&cfg, k_resident<ES>, P);
 }
 
-// The launch shape for blocks of nw warps (16: the one shape the engine uses) and element size es.
-cudaError_t resident_shape_for(int nw, int es, int C, int n, size_t smem, int *grid)
+// The launch shape for element size es.
+cudaError_t resident_shape_for(int es, int C, int n, size_t smem, int *grid)
 {
-    if (nw != kResMaxWarps) return cudaErrorInvalidValue;
-    return es == 2 ? resident_shape<kResMaxWarps, 2>(C, n, smem, grid) : resident_shape<kResMaxWarps, 1>(C, n, smem, grid);
+    return es == 2 ? resident_shape<2>(C, n, smem, grid) : resident_shape<1>(C, n, smem, grid);
 }
 
 }  // namespace
 
-// Largest cluster the device can run with blocks of nw warps and smem_limit
+// Largest cluster the device can run with blocks of smem_limit
 // bytes of shared memory each: 16 where clusters of 16 (a non-portable size)
 // can be resident, else 8.  Asked once per device.
-int resident_max_cluster(int nw, size_t smem_limit)
+int resident_max_cluster(size_t smem_limit)
 {
     static int cached[64] = {};
     int dev = 0;
@@ -748,8 +777,8 @@ int resident_max_cluster(int nw, size_t smem_limit)
     }
     if (!cached[dev]) {
         int g1 = 0, g2 = 0;
-        const cudaError_t e1 = resident_shape_for(nw, 1, kResMaxCluster, 1, smem_limit, &g1);
-        const cudaError_t e2 = resident_shape_for(nw, 2, kResMaxCluster, 1, smem_limit, &g2);
+        const cudaError_t e1 = resident_shape_for(1, kResMaxCluster, 1, smem_limit, &g1);
+        const cudaError_t e2 = resident_shape_for(2, kResMaxCluster, 1, smem_limit, &g2);
         cudaGetLastError();
         cached[dev] = (e1 == cudaSuccess && e2 == cudaSuccess && g1 == kResMaxCluster && g2 == kResMaxCluster)
                           ? kResMaxCluster
@@ -758,20 +787,19 @@ int resident_max_cluster(int nw, size_t smem_limit)
     return cached[dev];
 }
 
-// Smallest cluster (1, 2, 4, 8, or 16 where the device allows it, blocks of
-// nw warps) whose shared memory holds the image; 0 if none.
-int resident_cluster_size(int w, int h, int dtype, size_t smem_limit, int nw, int *rows_out, int *rp_out)
+// Smallest cluster (1, 2, 4, 8, or 16 where the device allows it) whose shared memory holds the image; 0 if none.
+int resident_cluster_size(int w, int h, int dtype, size_t smem_limit, int *rows_out, int *rp_out)
 {
     const int es = dtype == THIN_U16 ? 2 : 1;
     const int rp = int((size_t(w) * es + 15) / 16 * 16) + 32;
     const int cw = (w + 7) / 8, wpr = (cw + 31) / 32;
-    const int cmax = resident_max_cluster(nw, smem_limit);
+    const int cmax = resident_max_cluster(smem_limit);
     for (int C = 1; C <= cmax; C *= 2) {
         int rows = (h + C - 1) / C;
         rows += rows & 1;
         const int held = rows + (C > 1 ? 2 * std::min(kResStep, rows) : 0);  // halo: see resident_run
-        if (held / 2 * cw > 65535) continue;  // queue codes are 16-bit
-        if (res_smem_bytes(held, rp, wpr, nw) <= smem_limit) {
+        if (!codes_fit(held, cw)) continue;
+        if (res_smem_bytes(held, rp, wpr) <= smem_limit) {
             if (rows_out) *rows_out = rows;
             if (rp_out) *rp_out = rp;
             return C;
@@ -784,7 +812,7 @@ int resident_cluster_size(int w, int h, int dtype, size_t smem_limit, int nw, in
 // S (clusters) whose shared memory holds the image with all S clusters
 // resident at once (clusters must fit within a GPC, so large clusters cannot
 // use every SM).  Returns S and stores C, or 0 if none.
-int resident_wide_strips(int w, int h, int dtype, size_t smem_limit, int nw, int *c_out)
+int resident_wide_strips(int w, int h, int dtype, size_t smem_limit, int *c_out)
 {
     const int es = dtype == THIN_U16 ? 2 : 1;
     const int rp = int((size_t(w) * es + 15) / 16 * 16) + 32;
@@ -792,18 +820,18 @@ int resident_wide_strips(int w, int h, int dtype, size_t smem_limit, int nw, int
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int max_blocks = sms * (kResMaxWarps / nw);
+    const int max_blocks = sms;  // one block per SM
     for (int C = 8; C >= 1; C /= 2) {
         for (int S = 2; S * C <= max_blocks; ++S) {
             int rows = (h + S * C - 1) / (S * C);
             rows += rows & 1;
             const int held = rows + 2 * std::min(kResStep, rows);
-            if (held / 2 * cw > 65535) continue;  // queue codes are 16-bit
-            const size_t smem = res_smem_bytes(held, rp, wpr, nw);
+            if (!codes_fit(held, cw)) continue;
+            const size_t smem = res_smem_bytes(held, rp, wpr);
             if (smem > smem_limit) continue;
             // every cluster of the launch must be resident at once
             int grid = 0;
-            const cudaError_t e = resident_shape_for(nw, es, C, S, smem, &grid);
+            const cudaError_t e = resident_shape_for(es, C, S, smem, &grid);
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 return 0;
@@ -818,37 +846,32 @@ int resident_wide_strips(int w, int h, int dtype, size_t smem_limit, int nw, int
     return 0;
 }
 
-// Shared memory a block may take when `blocks` blocks share an SM.
-size_t resident_smem_limit(int blocks)
+// Shared memory a block may take (one block per SM).
+size_t resident_smem_limit()
 {
-    int dev = 0, optin = 0, per_sm = 0, reserved = 0;
+    int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-    size_t lim = size_t(optin > 0 ? optin : 48 * 1024);
-    if (blocks > 1 && per_sm > 0) lim = std::min(lim, size_t(per_sm) / blocks - size_t(reserved));
-    return lim;
+    return size_t(optin > 0 ? optin : 48 * 1024);
 }
 
 // Host-side preparation of one launch: job table (longest first), stats and
 // control words, and their pristine copies, all in one device allocation.
-int resident_prepare(const JobSpec *jobs, int n, int C, int nw, const thin_options &opt, cudaStream_t stream,
+int resident_prepare(const JobSpec *jobs, int n, int C, const thin_options &opt, cudaStream_t stream,
                      bool async_alloc, ResidentPrepared *R, int strips, ResDone *done)
 {
     *R = ResidentPrepared();
     R->n = n;
     R->C = C;
-    R->nw = nw;
     R->strips = strips;
     R->async_alloc = async_alloc;
     if (strips > 0 && n != 1) return THIN_ERR_ARG;  // a wide launch runs one image
     const int B = strips > 0 ? strips * C : C;      // blocks per image
-    if (nw != kResMaxWarps || n < 1) return THIN_ERR_ARG;
+    if (n < 1) return THIN_ERR_ARG;
     R->es = elem_size(jobs[0].dtype);
     for (int k = 1; k < n; ++k)
         if (elem_size(jobs[k].dtype) != R->es) return THIN_ERR_ARG;  // one element size per launch
-    const size_t limit = resident_smem_limit(kResMaxWarps / nw);
+    const size_t limit = resident_smem_limit();
     std::vector<ResJob> rj(n);
     size_t smem = 0;
     for (int k = 0; k < n; ++k) {
@@ -876,8 +899,8 @@ int resident_prepare(const JobSpec *jobs, int n, int C, int nw, const thin_optio
         r.adj = J.adj;
         r.done_slot = strips > 0 ? -1 : J.done_slot;
         const int held = r.rows + 2 * r.hr;
-        const size_t need = res_smem_bytes(held, r.rp, r.wpr, nw);
-        if (need > limit || held / 2 * r.cw > 65535) return THIN_ERR_ARG;
+        const size_t need = res_smem_bytes(held, r.rp, r.wpr);
+        if (need > limit || !codes_fit(held, r.cw)) return THIN_ERR_ARG;
         smem = std::max(smem, need);
     }
     // longest-first: larger lambda and larger images tend to run longer
@@ -894,7 +917,7 @@ int resident_prepare(const JobSpec *jobs, int n, int C, int nw, const thin_optio
 
     // launch shape first: time slices only pay when more jobs than clusters wait
     const int want = strips > 0 ? strips : n;  // clusters wanted
-    cudaError_t e = resident_shape_for(nw, R->es, C, want, smem, &R->grid);
+    cudaError_t e = resident_shape_for(R->es, C, want, smem, &R->grid);
     if (e != cudaSuccess) return cuda_status(e);
     if (strips > 0 && R->grid < B) return THIN_ERR_ARG;  // not all strips fit at once
     const int clusters = std::max(1, R->grid / C);
@@ -985,8 +1008,8 @@ cudaError_t resident_enqueue(const ResidentPrepared &R, cudaStream_t stream)
 {
     const cudaError_t e = cudaMemcpyAsync(R.live, R.pristine, R.live_bytes, cudaMemcpyDeviceToDevice, stream);
     if (e != cudaSuccess) return e;
-    return R.es == 2 ? resident_launch<kResMaxWarps, 2>(R.C, R.grid, R.smem, stream, R.P)
-                     : resident_launch<kResMaxWarps, 1>(R.C, R.grid, R.smem, stream, R.P);
+    return R.es == 2 ? resident_launch<2>(R.C, R.grid, R.smem, stream, R.P)
+                     : resident_launch<1>(R.C, R.grid, R.smem, stream, R.P);
 }
 
 // Waits for the stream and writes the stats of job k (the caller's order) to out[k].

@@ -385,7 +385,7 @@ int thin_serve_create(size_t device_budget_bytes, int max_slots, int queue_cap, 
         delete S;
         return THIN_ERR_CUDA;
     }
-    S->res_smem_limit = resident_smem_limit(1);
+    S->res_smem_limit = resident_smem_limit();
     // host staging for waiting and running requests: a quarter of the device
     // budget, between 256 MiB and 4 GiB
     const size_t host = std::min<size_t>(std::max<size_t>(device_budget_bytes / 4, size_t(256) << 20), size_t(4) << 30);
@@ -428,7 +428,7 @@ int thin_serve_submit(thin_server *S, const void *host_img, int w, int h, size_t
             return THIN_EAGAIN;
         }
     }
-    r->large = resident_cluster_size(w, h, dt, S->res_smem_limit, 16, nullptr, nullptr) == 0;
+    r->large = resident_cluster_size(w, h, dt, S->res_smem_limit, nullptr, nullptr) == 0;
     if (row * h > S->pool.size()) {
         delete r;
         return THIN_ERR_TOO_LARGE;  // could never be staged

@@ -86,7 +86,9 @@ struct PointRule {
     uint32_t tab;   // shared address of the decision table
     uint32_t mode;  // the decision's bit in a table entry
     uint32_t lam;   // lambda, capped at the largest difference of two pixels
-    bool cap;       // bound the marks by the old value + lambda (marks())
+    uint32_t lamh;  // lambda as two halves (u8 images)
+    float lamf;
+    bool cap;       // bound the marks by the old value + lambda (lower_item)
 };
 
 __device__ __forceinline__ PointRule point_rule(const void *table_smem, int mode, uint32_t lam, int es, bool cap)
@@ -95,6 +97,8 @@ __device__ __forceinline__ PointRule point_rule(const void *table_smem, int mode
     r.tab = static_cast<uint32_t>(__cvta_generic_to_shared(table_smem));
     r.mode = uint32_t(mode);
     r.lam = min(lam, es == 1 ? 255u : 65535u);
+    r.lamh = h2_from(min(r.lam, 255u));
+    r.lamf = float(r.lam);
     r.cap = cap;
     return r;
 }
@@ -192,9 +196,8 @@ struct Quad8 {
         add_below(nB, cB, loB, hiB);
         uint32_t base = R.tab - 0x6400u;
         if (R.lam != 0) {
-            const uint32_t lam = h2_from(R.lam);
-            add_below(nA, h2_sub(cA, lam), loA, hiA);
-            add_below(nB, h2_sub(cB, lam), loB, hiB);
+            add_below(nA, h2_sub(cA, R.lamh), loA, hiA);
+            add_below(nB, h2_sub(cB, R.lamh), loB, hiB);
         }
         // state index per lane, biased by 0x6400: lo + 81 hi
         uint32_t iA = (hiA & 0x00ff00ffu) * 81u + loA, iB = (hiB & 0x00ff00ffu) * 81u + loB;
@@ -241,8 +244,7 @@ struct Quad8 {
             sB = h2_fma(h2_subsat(nB[d], cB), h2_of(1 << d), sB);
         }
         if (R.cap) {
-            const uint32_t lam = h2_from(R.lam);
-            const uint32_t tA = h2_add(c0.A, lam), tB = h2_add(c0.B, lam);
+            const uint32_t tA = h2_add(c0.A, R.lamh), tB = h2_add(c0.B, R.lamh);
 #pragma unroll
             for (int d = 0; d < 8; ++d) {
                 sA = h2_fma(h2_subsat(nA[d], tA), h2_of(1 << d) | 0x80008000u, sA);
@@ -322,12 +324,11 @@ struct Quad16 {
 #pragma unroll
             for (int k = 0; k < 4; ++k) s[k] = __fmaf_rn(__saturatef(__fsub_rn(c[k], nb(k, d))), w[d], s[k]);
         if (R.lam != 0) {
-            const float lam = float(R.lam);
 #pragma unroll
             for (int d = 0; d < 8; ++d)
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    s[k] = __fmaf_rn(__saturatef(__fsub_rn(__fsub_rn(c[k], lam), nb(k, d))), w[d], s[k]);
+                    s[k] = __fmaf_rn(__saturatef(__fsub_rn(__fsub_rn(c[k], R.lamf), nb(k, d))), w[d], s[k]);
         }
         uint32_t t[4];
 #pragma unroll
@@ -369,12 +370,11 @@ struct Quad16 {
             for (int k = 0; k < 4; ++k)
                 s[k] = __fmaf_rn(__saturatef(__fsub_rn(nb(k, d), c[k])), float(1 << d), s[k]);
         if (R.cap) {
-            const float lam = float(R.lam);
 #pragma unroll
             for (int d = 0; d < 8; ++d)
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    s[k] = __fmaf_rn(__saturatef(__fsub_rn(nb(k, d), __fadd_rn(c0.v[k], lam))), -float(1 << d), s[k]);
+                    s[k] = __fmaf_rn(__saturatef(__fsub_rn(nb(k, d), __fadd_rn(c0.v[k], R.lamf))), -float(1 << d), s[k]);
         }
         const uint32_t a = __byte_perm(__float_as_uint(s[0]), __float_as_uint(s[1]), 0x0040);
         const uint32_t b = __byte_perm(__float_as_uint(s[2]), __float_as_uint(s[3]), 0x0040);
@@ -452,6 +452,51 @@ __device__ __forceinline__ uint32_t lower_item(const T *ra, T *rb, const T *rc, 
         if (MARK) aff = q.above(R, c0) & (moved * 0xffu);
     }
     return moved;
+}
+
+// One point on one lane: the same loop with the pixels as floats (either
+// element size), for phases with too few work items to fill the warps with
+// four points a lane.  A work item is then four lanes, and each of them issues
+// about a quarter of the instructions (a chain of one warp runs at the rate it
+// can issue: two cycles for each half-rate instruction).  ra, rb, rc point at
+// the point's column in rows y - 1, y and y + 1.  Returns the number of steps;
+// aff: the neighbours to test again, bit d for direction d.
+template <typename T>
+__device__ __forceinline__ int lower_one(const T *ra, T *rb, const T *rc, const PointRule &R, uint32_t &aff)
+{
+    constexpr uint32_t kBias = 0x4b000000u;  // 2^23
+    const float n[8] = {__uint_as_float(kBias | rb[1]),  __uint_as_float(kBias | ra[1]),  __uint_as_float(kBias | ra[0]),
+                        __uint_as_float(kBias | ra[-1]), __uint_as_float(kBias | rb[-1]), __uint_as_float(kBias | rc[-1]),
+                        __uint_as_float(kBias | rc[0]),  __uint_as_float(kBias | rc[1])};
+    const float c0 = __uint_as_float(kBias | rb[0]);
+    float c = c0;
+    constexpr float w[8] = {1, 3, 9, 27, 81, 243, 729, 2187};
+    int steps = 0;
+#pragma unroll 1
+    for (; steps < 9; ++steps) {
+        float s = __uint_as_float(kBias), t = 0.0f;
+        const float cl = __fsub_rn(c, R.lamf);
+        const uint32_t m = 0u - __float_as_uint(c);
+        uint32_t best = 0;
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            s = __fmaf_rn(__saturatef(__fsub_rn(c, n[d])), w[d], s);
+            t = __fmaf_rn(__saturatef(__fsub_rn(cl, n[d])), w[d], t);  // lambda = 0: all of them once more
+        }
+        const uint32_t e = lds_u8(R.tab + __float_as_uint(__fadd_rn(s, t)) - kBias);
+#pragma unroll
+        for (int d = 0; d < 8; ++d) best = __viaddmax_u32(__float_as_uint(n[d]), m, best);
+        if (!((e >> R.mode) & 1u)) break;
+        c = __uint_as_float(__float_as_uint(c) + best);
+    }
+    aff = 0;
+    if (steps) {
+        rb[0] = static_cast<T>(__float_as_uint(c));
+        const float top = R.cap ? __fadd_rn(c0, R.lamf) : __uint_as_float(0x4b800000u);  // above every pixel
+#pragma unroll
+        for (int d = 0; d < 8; ++d) aff |= n[d] > c && n[d] <= top ? 1u << d : 0u;
+    }
+    return steps;
 }
 
 }  // namespace thin
