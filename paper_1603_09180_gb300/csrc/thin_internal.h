@@ -175,7 +175,12 @@ cudaError_t tiled_enqueue(const TiledPrepared *T, cudaStream_t stream);
 int tiled_collect(const TiledPrepared *T, const thin_options &opt, cudaStream_t stream, thin_stats *out);
 void tiled_release(TiledPrepared *T, cudaStream_t stream);
 
-// Defaults of the tiled engine for a dtype (tile width/height in pixels, halo).
+// The shape the tiled engine takes by itself for these images; true if they are
+// enough for its large tiles to fill the GPU (nothing to tune then).
+bool tiled_fills(const JobSpec *jobs, int n, int *tw, int *th, int *H);
+
+// Defaults of the tiled engine for a dtype (tile width/height in pixels, halo)
+// where the caller sets only some of them.
 void tiled_defaults(int dtype, int *tw, int *th, int *halo);
 
 int cuda_status(cudaError_t e);

@@ -108,24 +108,30 @@ int thin_plan_create(const thin_job *jobs, int n, thin_adj adj, const thin_optio
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
     for (auto &x : ev)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
-    // The tiled group's tile shape and halo depth: autotuned on its largest
-    // image (trials on a scratch copy, 64 phases each) unless the caller set them.
+    // The tiled group's tile shape and halo depth: where its large tiles do not
+    // fill the GPU, autotuned on its largest image (trials on a scratch copy, 64
+    // phases each), unless the caller set them.
     thin_options ot = o;
+    int fill_w = 0, fill_h = 0, fill_halo = 0;
     if (e == cudaSuccess && !G.tiled.empty() && o.tile_w == 0 && o.tile_h == 0 && o.halo == 0) {
         int big = G.tiled[0];
         for (int k : G.tiled)
             if (double(p->specs[k].w) * p->specs[k].h > double(p->specs[big].w) * p->specs[big].h) big = k;
         const JobSpec &J = p->specs[big];
         thin_options tuned = o;
-        if (thin_autotune(J.img, J.w, J.h, J.pitch, thin_dtype(J.dtype), J.lam, cs, 64, &tuned, nullptr) == THIN_OK) {
+        std::vector<JobSpec> js;
+        for (int k : G.tiled) js.push_back(p->specs[k]);
+        if (tiled_fills(js.data(), int(js.size()), &fill_w, &fill_h, &fill_halo)) {
+            // the engine's own choice for the whole group
+        } else if (thin_autotune(J.img, J.w, J.h, J.pitch, thin_dtype(J.dtype), J.lam, cs, 64, &tuned, nullptr) == THIN_OK) {
             // a u16 image in the group caps the halo at 8; autotune tried that image's dtype only
             bool any16 = false;
             for (int k : G.tiled) any16 |= p->specs[k].dtype == THIN_U16;
             if (!any16 || tuned.halo <= 8) ot = tuned;
         }
-        p->tile_w = ot.tile_w;
-        p->tile_h = ot.tile_h;
-        p->halo = ot.halo;
+        p->tile_w = ot.tile_w ? ot.tile_w : fill_w;
+        p->tile_h = ot.tile_w ? ot.tile_h : fill_h;
+        p->halo = ot.tile_w ? ot.halo : fill_halo;
     }
     if (e == cudaSuccess) {
         rc = p->X.prepare(p->specs, G, ot, cs, true);  // plan-owned device memory, stream-ordered on cs

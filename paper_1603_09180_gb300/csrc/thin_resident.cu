@@ -51,6 +51,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "thin_block.cuh"
 #include "thin_common.cuh"
 #include "thin_internal.h"
 #include "thin_simd.cuh"
@@ -64,11 +65,6 @@ namespace {
 // Warps per block, one block per SM (at most 128 registers a thread).
 constexpr int kResWarps = 16;
 constexpr int kResThreads = 32 * kResWarps;
-// Phases with at most this many groups in a block take a lane to a point (four
-// to a group): 64^2 at lambda = 10 245 -> 220 us, 192 512^2 u16 images
-// 24.1 -> 23.9 ms; at 256 a block's lanes take two turns, and the u8 batch lost
-// 3 %.
-constexpr int kLaneItems = 128;
 constexpr int kResStep = 8;  // phases between halo exchanges = halo rows held from each neighbour
 __device__ const DecisionTable d_res_decisions = kDecisionTable;
 
@@ -229,12 +225,6 @@ __device__ void res_push(const ResArgs &P, int job)
     *reinterpret_cast<volatile unsigned *>(&P.tag[s]) = 1u + t / P.cap;
 }
 
-// ORs m into a word of shared memory; nothing where m is 0 (a predicate, not a branch).
-__device__ __forceinline__ void smem_or(uint32_t addr, uint32_t m)
-{
-    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %1, 0;\n @p red.shared.or.b32 [%0], %1;\n}\n" ::"r"(addr), "r"(m) : "memory");
-}
-
 // ES: element size of every image of the launch (1: u8, 2: u16).
 template <int ES>
 __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs P)
@@ -289,7 +279,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs P)
         uint32_t *dirty = reinterpret_cast<uint32_t *>(smem + res_bits_off(LR, RP));
         // the block's queue of the groups found in one scan round
         uint16_t *bqueue = reinterpret_cast<uint16_t *>(smem + res_queue_off(LR, RP, WPR));
-        const uint32_t dirty_s = res_smem_u32(dirty);
         const int row0 = gb * R;         // first own image row
         const int ybase = row0 - HR;     // image row of shared row 0
         const int rowb = J.w * es;
@@ -357,8 +346,17 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs P)
         // decisions and their cluster barriers stop pairing.
         cluster.sync();
 
-        // A group's code is (cell row << cbits) | cell column.
-        const int cbits = 32 - __clz(CW - 1);
+        PieceMap map;
+        map.rows = rows_base + 16;
+        map.dirty = res_smem_u32(dirty);
+        map.pitch = RP;
+        map.cell_words = WPR;
+        map.bitmap_words = slot_words;
+        map.cbits = 32 - __clz(CW - 1);
+        map.own_row = HC;
+        map.own_rows = R / 2;
+        map.own_col = 0;
+        map.own_cols = CW;
         // This thread's piece of a bitmap: the word, where its bits lie, the columns that exist, the
         // code of its first group.  It stays the same for the whole job unless the bitmap needs several
         // scan rounds.
@@ -373,7 +371,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs P)
             const int cc = (pword - prow * WPR) * 32 + pshift;
             const int valid = min(CW - cc, 8 << unit);
             pmask = pword >= slot_words || valid <= 0 ? 0u : valid >= 32 ? 0xffffffffu : (1u << valid) - 1u;
-            pcode = (prow << cbits) | cc;
+            pcode = (prow << map.cbits) | cc;
         };
         take_piece(0);
 
@@ -390,42 +388,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs P)
             for (int j = 0; j < Hs; ++j, ++g) {
                 const int p = int(g & 3), px = p & 1, py = p >> 1;
                 uint32_t *dp = dirty + p * slot_words;
-                // the groups of the other three parities holding a neighbour to test again become
-                // dirty.  A: byte k holds the ring directions (bit 0 E, 1 NE, 2 N, 3 NW, 4 W, 5 SW,
-                // 6 S, 7 SE) of point k's neighbours to mark; 0: nothing to mark.  E and W neighbours
-                // are in the row's other column parity, N and S in the other row parity, the
-                // diagonals in the fourth.  For px == 0 the W side of point 0 is in the cell to the
-                // left; for px == 1 the E side of point 3 is in the cell to the right.
-                const uint32_t pbytes = 4u * uint32_t(slot_words), up = py ? 0u : 0u - 4u * uint32_t(WPR);
-                const uint32_t qrow = pbytes * uint32_t(2 * py + (px ^ 1)), qcol = pbytes * uint32_t(2 * (py ^ 1) + px) + up,
-                               qdiag = pbytes * uint32_t(2 * (py ^ 1) + (px ^ 1)) + up;
-                auto mark = [&](int cr, int cc, uint32_t A) {
-                    const uint32_t beside = px ? 0x83000000u : 0x00000038u;  // towards the cell beside
-                    const uint32_t X = A & beside, x = px ? X >> 24 : X;
-                    uint32_t f = A ^ X;  // the rest, folded into one set of directions
-                    f |= f >> 16;
-                    f |= f >> 8;
-                    const uint32_t mc = 1u << (cc & 31);
-                    const uint32_t mx = px ? mc << 1 : mc >> 1;  // 0: the cell beside is in the next word
-                    const uint32_t mrow = (f & 0x11u ? mc : 0u) | (x & 0x11u ? mx : 0u);
-                    const uint32_t ma = (f & 0x0au ? mc : 0u) | (x & 0x0au ? mx : 0u);
-                    const uint32_t mb = (f & 0xa0u ? mc : 0u) | (x & 0xa0u ? mx : 0u);
-                    // word of the group's own cell in the bitmap of each parity; of the cell row of y - 1
-                    const uint32_t o = dirty_s + 4u * uint32_t(cr * WPR + (cc >> 5));
-                    const uint32_t drow = o + qrow, dcol = o + qcol, ddiag = o + qdiag;
-                    const uint32_t below = 4u * uint32_t(WPR);
-                    smem_or(drow, mrow);
-                    smem_or(dcol, f & 0x04u ? mc : 0u);
-                    smem_or(ddiag, ma);
-                    smem_or(dcol + below, f & 0x40u ? mc : 0u);
-                    smem_or(ddiag + below, mb);
-                    if (mx == 0u && x) {  // the group across a word boundary (rare)
-                        const uint32_t ws = px ? 4u : ~3u, ms = px ? 1u : 0x80000000u;
-                        smem_or(drow + ws, x & 0x11u ? ms : 0u);
-                        smem_or(ddiag + ws, x & 0x0au ? ms : 0u);
-                        smem_or(ddiag + below + ws, x & 0xa0u ? ms : 0u);
-                    }
-                };
                 bool moved_own = false;
                 // A scan round: each thread takes one piece of the parity's bitmap (a byte, or 16 or
                 // 32 bits where there are more of them than threads), consumes its bits and appends the
@@ -460,45 +422,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident(ResArgs P)
                     const int N = int(*reinterpret_cast<volatile unsigned *>(&ctrl->qn[qround & 1]));
                     if (tid == 0) ctrl->qn[(qround + 1) & 1] = 0u;  // last read in the previous round
                     ++qround;
-                    if (N <= kLaneItems) {
-                        // few groups: a lane to a point
-                        for (int k = tid >> 2; k < N; k += kResThreads / 4) {
-                            const int code = bqueue[k], j4 = lane & 3;
-                            const int cr = code >> cbits, cc = code - (cr << cbits);
-                            const int x = 8 * cc + px + 2 * j4;
-                            if (x >= 1 && x <= J.w - 2) {
-                                T *rb = reinterpret_cast<T *>(rows_base + (2 * cr + py) * RP + 16) + x;
-                                const T *ra = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) - RP);
-                                const T *rc = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) + RP);
-                                uint32_t A;
-                                const int n = lower_one<T>(ra, rb, rc, rule, A);
-                                if (unsigned(cr - HC) < unsigned(R / 2)) {  // own rows count
-                                    ++ntest;
-                                    nlow += n;
-                                    moved_own |= n > 0;
-                                }
-                                if (A) mark(cr, cc, A << (8 * j4));
-                            }
-                        }
-                    } else {
-                        // Chunks of 32 groups go to the warps in turn: every chunk but the last is full, and
-                        // the schedulers' shares differ by one chunk at most.
-                        for (int k = tid; k < N; k += kResThreads) {
-                            const int code = bqueue[k];
-                            const int cr = code >> cbits, cc = code - (cr << cbits);
-                            const int last = (J.w - 2 - px - 8 * cc) >> 1;  // last point inside the image border
-                            uint32_t vm = last >= 3 ? kLsb8 : last >= 0 ? kLsb8 >> (8 * (3 - last)) : 0u;
-                            if (px == 0 && cc == 0) vm &= ~1u;  // x = 0
-                            const uint32_t in = unsigned(cr - HC) < unsigned(R / 2) ? vm : 0u;  // own rows count
-                            ntest += int((in * kLsb8) >> 24);
-                            T *rb = reinterpret_cast<T *>(rows_base + (2 * cr + py) * RP + 16) + 8 * cc;
-                            const T *ra = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) - RP);
-                            const T *rc = reinterpret_cast<const T *>(reinterpret_cast<const uint8_t *>(rb) + RP);
-                            uint32_t aff;
-                            moved_own |= (lower_item<true>(ra, rb, rc, px, vm, in, rule, nlow, aff) & in) != 0;
-                            if (aff) mark(cr, cc, aff);
-                        }
-                    }
+                    moved_own |= work_queue<T, kResThreads>(map, rule, bqueue, N, px, py, 1, J.w - 2, nlow, ntest);
                     if (r0 + kScanWords < slot_words) __syncthreads();  // the next round refills the queue
                 }
                 if (moved_own) ctrl->last = g;  // (every writer writes the same value)

@@ -429,7 +429,7 @@ struct QuadOf<uint16_t> {
 // which saves more tests than it costs in a batch but not in the wide mode's
 // tail.  This holds in every mode, since the decision depends on the
 // neighbour values through those two masks only.
-template <bool MARK, typename T>
+template <typename T>
 __device__ __forceinline__ uint32_t lower_item(const T *ra, T *rb, const T *rc, int px, uint32_t vm, uint32_t in,
                                                const PointRule &R, int &nin, uint32_t &aff)
 {
@@ -449,7 +449,7 @@ __device__ __forceinline__ uint32_t lower_item(const T *ra, T *rb, const T *rc, 
     aff = 0;
     if (moved) {
         q.store(rb, px);
-        if (MARK) aff = q.above(R, c0) & (moved * 0xffu);
+        aff = q.above(R, c0) & (moved * 0xffu);
     }
     return moved;
 }

@@ -3,30 +3,37 @@
 // One persistent cooperative launch runs the whole subfield schedule for any
 // number of images.  The schedule advances in steps of H phases (temporal
 // blocking).  In a step every active tile of every image is visited by one
-// warp: a TMA 2-D tile load stages the tile with a halo of H pixels in the
-// warp's shared memory, the warp advances H consecutive phases there (the exact
-// region shrinks by one pixel ring per phase, so the TW x TH interior is exact
-// after H phases) and stores the interior to the other buffer of a ping-pong
-// pair.  A grid barrier separates steps.
+// block: TMA 2-D tile loads stage the tile with a halo in shared memory, the
+// block advances H consecutive phases there (the exact region shrinks by one
+// pixel ring per phase) and stores the interior to the other buffer of a
+// ping-pong pair.  A grid barrier separates steps.
 //
-// Which points a phase must test.  A point whose 8 neighbours did not change
-// since its own last test (four phases earlier) cannot have become
-// lambda-destructible, so skipping it changes nothing.  Changes are recorded
-// per cell of 8 x 2 pixels as the global index of the last phase that lowered
-// a point in the cell; these stamps persist per image between tile visits.  A
-// group of four points is tested at phase g only if a cell of its 3 x 3 cell
-// neighbourhood changed at a phase >= g - 3.  Stamps start at the first phase
-// of the run, so every point is tested during the first four phases.
+// Which points a phase tests.  As in the resident engine (thin_block.cuh): per
+// parity a dirty bit per 4-point group, set by the moves of its neighbours that
+// can change its test, consumed by its phase.  Between visits the bits of an
+// image lie in global memory, a byte per cell with a bit per parity, in a
+// ping-pong pair of their own: a visit reads the bits of its tile and halo as
+// they were at the start of the step and writes those of its tile.  The halo is
+// one pixel wider than the step has phases, so that in the last phase too the
+// points just outside the tile are exact: every mark a neighbour's move makes
+// inside the tile is made by the tile's own visit, and no visit writes another
+// tile's bits.
 //
-// Which tiles a step visits.  At the start of a step (phase g0) every unstable
-// point lies next to a point that changed during phases g0-3 .. g0-1, and
-// unstable points spread by at most one pixel per phase, so a tile none of
-// whose 3x3 block of tiles changed in those three phases cannot change during
-// the next H <= min(TW, TH) - 1 phases: it is skipped.  A tile that changed at
-// all in a step is also visited in the next one, which keeps both ping-pong
-// buffers equal on every skipped tile.  The first step (and any step starting
-// within three phases of the first) visits every tile.  When a step visits no
-// tile the image is at its fixed point and both buffers hold it.
+// Which tiles a step visits.  A tile that changed at all, which keeps both
+// ping-pong buffers equal on every skipped tile; a tile with a dirty bit; and
+// its neighbours as far as a move of such a bit's group can come in H phases (a
+// move spreads one pixel a phase).  The first step visits every tile, with every
+// bit set.  When a step visits no tile the image is at its fixed point and both
+// buffers hold it.
+//
+// What bounds it: issue, as in the resident engine (8192^2 u16 at lambda = 0 is
+// read and written once in each of 9 steps: 2.4 GB, 0.4 of 4.8 ms).  Tiles were
+// 64 x 32 pixels, one to a warp, with change stamps that re-tested every group
+// of the nine cells around a changed one: a ring of 8 around such a tile is a
+// third more points, and the stamps' scan took 300 instructions a phase.
+// 8192^2 u16 went from 7.1 to 4.8 ms at lambda = 0 and from 22.5 to 13.9 ms at
+// lambda = 30; 1024 uneven u8 images from 277 to 239 ms; 48 served requests of
+// every size from 91 to 46 ms.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -37,6 +44,7 @@
 #include <mutex>
 #include <vector>
 
+#include "thin_block.cuh"
 #include "thin_common.cuh"
 #include "thin_internal.h"
 #include "thin_simd.cuh"
@@ -48,6 +56,8 @@ namespace {
 constexpr int kWarps = 8;
 constexpr int kThreads = 32 * kWarps;
 constexpr int kMinHalo = 3;
+constexpr int kPadCols = 16;   // halo columns staged on each side of a tile (two cells)
+constexpr int kMaxStep = 15;   // phases a step can have: one halo column more than that is needed
 
 struct ImgDesc {
     CUtensorMap map[2];          // TMA descriptors of buffer 0 and buffer 1
@@ -55,7 +65,7 @@ struct ImgDesc {
     unsigned long long pitch;    // row pitch of both buffers, bytes
     unsigned long long user;     // caller's image
     unsigned long long user_pitch;
-    unsigned long long cells;    // int32 stamps, cells_x x cells_y, relative to the first phase
+    unsigned long long cells[2]; // dirty bits of the ping-pong pair: a byte per cell, bit p for parity p
     int w, h, dtype;
     unsigned lam;
     int tiles_x, tiles_y, tile_base, copy_in;
@@ -80,16 +90,18 @@ struct Ctl {
     unsigned next_item[3];  // per step (mod 3): items claimed beyond the first one of every warp
 };
 
-// Shared memory of one warp: tile buffer, cell stamps (with a border ring of
-// never-changing cells), work queue and mbarrier.
-struct WarpLayout {
-    int tile_bytes;   // TMA box bytes + 16 (word reads past the last row stay inside)
-    int cell_off;     // offset of the stamps
-    int queue_off;    // offset of the queue (u16 entries)
-    int bar_off;      // offset of the mbarrier
-    int bytes;        // total, 128-aligned
-    int ccols, crows; // stamp grid including the border ring
+// Shared memory of a block: decision table, control words, tile rows, dirty
+// bitmaps (a word per cell row and parity: a tile and its halo are at most 32
+// cells wide), queue of groups.
+struct TileLayout {
+    int row_bytes;   // bytes of a staged row (tile and halo columns)
+    int rows;        // staged rows
+    int box_rows;    // rows of one TMA box (one or two boxes to a tile)
+    int dirty_off, queue_off, bytes;
 };
+constexpr int kOffCtrl = (kDecisionBytes + 15) / 16 * 16;  // control words, then the mbarrier
+constexpr int kOffBar = kOffCtrl + 32;
+constexpr int kOffTile = (kOffBar + 8 + 127) / 128 * 128;  // TMA destinations are 128-byte aligned
 
 struct EngineArgs {
     const ImgDesc *imgs;
@@ -99,11 +111,11 @@ struct EngineArgs {
     Ctl *ctl;
     int n_imgs;
     int total_tiles;
-    int tw, th, halo, hr, rule;  // hr: halo rows in shared memory (halo rounded up to even)
+    int tw, th, halo, hr, rule;  // halo: phases per step; hr: halo rows staged above and below (even, more than halo)
     long long start_phase;
     long long max_phases;
     unsigned long long timeout_ns;
-    WarpLayout wl;
+    TileLayout tl;
     int debug;         // 1: block 0 never arrives at the first barrier (timeout test)
 };
 
@@ -148,10 +160,8 @@ __device__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long time
     }
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar,
-                                            uint32_t bytes)
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar)
 {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
         "[%4];" ::"r"(dst),
@@ -226,116 +236,101 @@ __device__ __forceinline__ uint32_t div_magic(int d)
     return d > 1 ? 0xffffffffu / uint32_t(d) + 1u : 0u;
 }
 
-// Per-visit constants, held in registers.
+// One visit of a block: the tile, its place in the image and the step.
 struct Visit {
     int w, h;           // image size
-    uint32_t lam;
-    int rule;
     int x0, y0;         // tile origin in the image
     int tw, th;         // tile size
-    int H, Hs, hr;      // halo, phases to run, halo rows in shared memory
-    int pad;            // elements of left pad in shared memory (16 B)
+    int Hs, hr;         // phases to run, halo rows staged
     long long g0;       // global index of the first phase of the step
-    long long start;    // global index of the first phase of the run
 };
 
-// Hs phases of the subfield schedule on a staged tile, visited by one warp.
-// Shared cell (sx, sy) holds image pixel (x0 - pad + sx, y0 - hr + sy); stamp
-// cell (cx, cy) of the grid covers shared columns 8 (cx - 1) .. + 7 and rows
-// 2 (cy - 1) .. + 1 (one border ring of never-changing cells).  Phase j updates
-// the points of its parity within distance Hs-1-j of the tile and off the
-// image border; after Hs phases the tile interior is exact.
+// The block's control words.
+struct TileCtrl {
+    unsigned qn[2];     // fill counters of the queue, alternating by phase
+    unsigned next;      // the next list entry to visit
+    unsigned near;      // bit 3 (dy + 1) + dx + 1: the tile at (dx, dy) may change next step
+    int last;           // last phase of the step that moved a point of the tile, -1 none
+};
+static_assert(sizeof(TileCtrl) <= kOffBar - kOffCtrl, "control words overlap the mbarrier");
+
+// Hs phases of the subfield schedule on a staged tile.  Staged column 0 is
+// image column x0 - kPadCols, staged row 0 image row y0 - hr.  Phase j updates
+// the points of its parity within distance Hs - j of the tile and off the image
+// border; after Hs phases the tile and its dirty bits are exact.
 template <typename T>
-__device__ void visit_phases(T *tile, int bw, uint8_t *cells, int ccols, uint16_t *queue, const Visit &V,
-                             const uint8_t *tab, int &nlow, int &chg_j, int &ntest)
+__device__ __forceinline__ void visit_phases(const TileLayout &L, uint8_t *smem, const Visit &V, const PointRule &rule,
+                                             int &nlow, int &ntest, int &chg_j)
 {
-    const PointRule rule = point_rule(tab, V.rule, V.lam, sizeof(T), false);
-    const int lane = threadIdx.x & 31;
-    const unsigned lt_lanes = (1u << lane) - 1u;
+    TileCtrl *ctrl = reinterpret_cast<TileCtrl *>(smem + kOffCtrl);
+    uint32_t *dirty = reinterpret_cast<uint32_t *>(smem + L.dirty_off);
+    uint16_t *queue = reinterpret_cast<uint16_t *>(smem + L.queue_off);
+    const int words = L.rows / 2;
+    PieceMap map;
+    map.rows = smem + kOffTile;
+    map.dirty = smem_u32(dirty);
+    map.pitch = L.row_bytes;
+    map.cell_words = 1;
+    map.bitmap_words = words;
+    map.cbits = 5;
+    map.own_row = V.hr / 2;
+    map.own_rows = V.th / 2;
+    map.own_col = kPadCols / 8;
+    map.own_cols = V.tw / 8;
+    // this thread's piece of a bitmap: a byte, or 16 or 32 bits where there are more of them than threads
+    const int unit = words * 4 <= kThreads ? 0 : words * 2 <= kThreads ? 1 : 2;
+    const int pword = int(threadIdx.x) >> (2 - unit), pshift = (int(threadIdx.x) << (3 + unit)) & 31;
+    const uint32_t pones = unit == 0 ? 0xffu : unit == 1 ? 0xffffu : 0xffffffffu;
     for (int j = 0; j < V.Hs; ++j) {
-        const long long g = V.g0 + j;
-        const int p = int(g & 3);
-        const int px = p & 1, py = p >> 1;
-        const int r = V.Hs - 1 - j;
-        const int lox = max(V.x0 - r, 1), hix = min(V.x0 + V.tw + r - 1, V.w - 2);
-        const int loy = max(V.y0 - r, 1), hiy = min(V.y0 + V.th + r - 1, V.h - 2);
-        const int ya = loy + ((py - loy) & 1);
-        const int nrows = hiy >= ya ? (hiy - ya) / 2 + 1 : 0;
-        const int slo = lox - V.x0 + V.pad, shi = hix - V.x0 + V.pad;
-        const int qlo = slo >> 3;
-        const int nq = shi >= slo ? (shi >> 3) - qlo + 1 : 0;
-        const uint32_t Mq = div_magic(nq);
-        const int sra = ya - V.y0 + V.hr;
-        const int items = nrows * nq;
-        // 1. the items whose 3x3 stamp cells changed in the last three phases
-        int qn = 0;
-        for (int base = 0; base < items; base += 32) {
-            const int it = base + lane;
-            bool dirty = false;
-            int code = 0;
-            if (it < items) {
-                const int rk = div_small(it, nq, Mq);
-                const int q = qlo + it - rk * nq;
-                const int sr = sra + 2 * rk;
-                const uint8_t *cp = cells + ((sr >> 1) + 1) * ccols + q + 1;
-                uint32_t m = max(max(uint32_t(cp[-ccols - 1]), uint32_t(cp[-ccols])), uint32_t(cp[-ccols + 1]));
-                m = max(m, max(max(uint32_t(cp[-1]), uint32_t(cp[0])), uint32_t(cp[1])));
-                m = max(m, max(max(uint32_t(cp[ccols - 1]), uint32_t(cp[ccols])), uint32_t(cp[ccols + 1])));
-                dirty = m > uint32_t(j);  // a stamp of phase g - 3 or later
-                code = (sr << 6) | q;
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, dirty);
-            if (dirty) queue[qn + __popc(bal & lt_lanes)] = uint16_t(code);
-            qn += __popc(bal);
-        }
-        __syncwarp();
-        // 2. test and lower them
-        bool chg = false;
-        for (int k = lane; k < qn; k += 32) {
-            const int code = queue[k];
-            const int sr = code >> 6, q = code & 63, sb = 8 * q;
-            uint32_t vm = 0;
+        const int p = int((V.g0 + j) & 3), px = p & 1, py = p >> 1;
+        const int r = V.Hs - j;
+        const int xlo = max(V.x0 - r, 1) - V.x0 + kPadCols, xhi = min(V.x0 + V.tw - 1 + r, V.w - 2) - V.x0 + kPadCols;
+        if (pword < words) {
+            uint32_t *dp = dirty + p * words;
+            uint32_t d = (dp[pword] >> pshift) & pones;
+            if (d) {
+                if (unit == 0) reinterpret_cast<uint8_t *>(dp)[threadIdx.x] = 0;
+                else if (unit == 1) reinterpret_cast<uint16_t *>(dp)[threadIdx.x] = 0;
+                else dp[threadIdx.x] = 0;
+                const int y = V.y0 - V.hr + 2 * pword + py;
+                const uint32_t cols = (0xffffffffu << (xlo >> 3)) & (0xffffffffu >> (31 - (xhi >> 3)));
+                d &= cols >> pshift;
+                if (d && y >= max(V.y0 - r, 1) && y <= min(V.y0 + V.th - 1 + r, V.h - 2)) {
+                    uint16_t *q = queue + atomicAdd(&ctrl->qn[j & 1], unsigned(__popc(d)));
+                    int code = (pword << 5) | pshift;
+                    do {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                vm |= (unsigned(sb + px + 2 * kk - slo) <= unsigned(shi - slo) ? 1u : 0u) << (8 * kk);
-            const bool inside = unsigned(sr - V.hr) < unsigned(V.th) && sb >= V.pad && sb < V.pad + V.tw;
-            const uint32_t in = inside ? vm : 0u;
-            ntest += __popc(in);
-            uint32_t aff;  // (this engine marks whole cells: aff is not used)
-            T *rb = tile + sr * bw + sb;
-            const uint32_t moved = lower_item<false>(rb - bw, rb, rb + bw, px, vm, in, rule, nlow, aff);
-            if (moved) {
-                cells[((sr >> 1) + 1) * ccols + q + 1] = uint8_t(j + 4);
-                if (moved & in) chg = true;
+                        for (int b = 0; b < 8; ++b)
+                            if ((d >> b) & 1u) *q++ = uint16_t(code + b);
+                        code += 8;
+                        d >>= 8;
+                    } while (d);
+                }
             }
         }
-        if (__any_sync(0xffffffffu, chg)) chg_j = j;
-        __syncwarp();
+        __syncthreads();
+        const int N = int(*reinterpret_cast<volatile unsigned *>(&ctrl->qn[j & 1]));
+        if (threadIdx.x == 0) ctrl->qn[(j + 1) & 1] = 0u;  // last read in the previous phase
+        if (work_queue<T, kThreads>(map, rule, queue, N, px, py, xlo, xhi, nlow, ntest)) chg_j = j;
+        __syncthreads();
     }
 }
 
-// Store the tile interior (clipped to the image) to `dst`; 16 bytes of left pad.
-__device__ void tile_store(const uint8_t *tile, int bw_bytes, int es, const Visit &V, char *dst, size_t pitch)
+// Stores the tile (clipped to the image) to `dst`, a row of which is 16-byte aligned.
+__device__ __forceinline__ void tile_store(const uint8_t *tile, int row_bytes, int es, const Visit &V, char *dst, size_t pitch)
 {
-    const int lane = threadIdx.x & 31;
     const int cw = min(V.tw, V.w - V.x0) * es, ch = min(V.th, V.h - V.y0);
-    const int rowb = V.tw * es;
+    const int vpr = (cw + 15) / 16;
+    const uint32_t M = div_magic(vpr);
     char *base = dst + size_t(V.y0) * pitch + size_t(V.x0) * es;
-    const uint8_t *src = tile + V.hr * bw_bytes + 16;
-    if (cw == rowb) {
-        const int vpr = rowb / 16;
-        const uint32_t Mv = div_magic(vpr);
-        for (int v = lane; v < ch * vpr; v += 32) {
-            const int row = div_small(v, vpr, Mv), col = v - row * vpr;
-            *reinterpret_cast<uint4 *>(base + size_t(row) * pitch + col * 16) =
-                *reinterpret_cast<const uint4 *>(src + row * bw_bytes + col * 16);
-        }
-    } else {
-        const uint32_t Mc = div_magic(cw);
-        for (int e = lane; e < ch * cw; e += 32) {
-            const int row = div_small(e, cw, Mc), col = e - row * cw;
-            base[size_t(row) * pitch + col] = char(src[row * bw_bytes + col]);
-        }
+    const uint8_t *src = tile + V.hr * row_bytes + kPadCols * es;
+    for (int v = threadIdx.x; v < ch * vpr; v += kThreads) {
+        const int row = div_small(v, vpr, M), col = (v - row * vpr) * 16;
+        char *d = base + size_t(row) * pitch + col;
+        const uint8_t *s = src + row * row_bytes + col;
+        if (col + 16 <= cw) *reinterpret_cast<uint4 *>(d) = *reinterpret_cast<const uint4 *>(s);
+        else
+            for (int b = 0; col + b < cw; ++b) d[b] = char(s[b]);
     }
 }
 
@@ -350,25 +345,21 @@ __device__ __forceinline__ void decode(const EngineArgs &P, bool full, const uns
     tx = local - ty * D.tiles_x;
 }
 
-constexpr int kSmemTabs = (kDecisionBytes + 127) / 128 * 128;  // the decision table
-
 __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
 {
     extern __shared__ __align__(128) uint8_t smem_raw[];
-    // TMA destinations want 128-byte aligned shared addresses
     uint8_t *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    const uint8_t *tabs = smem;
     __shared__ int s_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const WarpLayout WL = P.wl;
-    uint8_t *wbase = smem + kSmemTabs + warp * WL.bytes;
-    uint8_t *tile = wbase;
-    uint8_t *cells = wbase + WL.cell_off;
-    uint16_t *queue = reinterpret_cast<uint16_t *>(wbase + WL.queue_off);
-    const uint32_t bar = smem_u32(wbase + WL.bar_off);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const TileLayout L = P.tl;
+    uint8_t *tile = smem + kOffTile;
+    TileCtrl *ctrl = reinterpret_cast<TileCtrl *>(smem + kOffCtrl);
+    uint32_t *dirty = reinterpret_cast<uint32_t *>(smem + L.dirty_off);
+    const uint32_t bar = smem_u32(smem + kOffBar);
+    const int words = L.rows / 2;
 
     load_decisions(smem, d_decisions);
-    if (lane == 0) {
+    if (tid == 0) {
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -377,119 +368,121 @@ __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
     uint32_t parity = 0;
     long long g0 = P.start_phase;
     const int H = P.halo, HR = P.hr;
-    const unsigned nwarps = gridDim.x * kWarps;
-    // consecutive items go to different blocks first, so that a step with few
-    // tiles spreads them over the SMs instead of stacking them on one
-    const unsigned gw = warp * gridDim.x + blockIdx.x;
-    const uint32_t Mcc = div_magic(WL.ccols);
     for (int s = 0;; ++s) {
         const long long done = g0 - P.start_phase;
         const int Hs = (P.max_phases >= 0 && P.max_phases - done < H) ? int(P.max_phases - done) : H;
-        const bool full = done <= 3;
+        const bool full = s == 0;
         const unsigned count = full ? unsigned(P.total_tiles)
                                     : *reinterpret_cast<volatile unsigned *>(&P.ctl->list_count[s % 3]);
-        const unsigned *L = P.lists + size_t(s % 3) * P.total_tiles;
+        const unsigned *Lcur = P.lists + size_t(s % 3) * P.total_tiles;
         unsigned *Lnext = P.lists + size_t((s + 1) % 3) * P.total_tiles;
-        if (blockIdx.x == 0 && threadIdx.x == 0) {  // counters of step s + 2, last used in step s - 1
+        if (blockIdx.x == 0 && tid == 0) {  // counters of step s + 2, last used in step s - 1
             P.ctl->list_count[(s + 2) % 3] = 0;
             P.ctl->next_item[(s + 2) % 3] = 0;
         }
         const int src = s & 1;
         bool failed = false;
-        // Every warp takes item gw first, then claims further items one at a time from the step's counter,
-        // so that warps that drew light tiles take more of them and the step ends with the grid together.
-        for (unsigned i = gw; i < count;) {
+        // A block takes item blockIdx.x first, then claims further items one at a time from the step's
+        // counter, so that blocks that drew light tiles take more of them.
+        for (unsigned i = blockIdx.x; i < count;) {
             int img, tx, ty;
-            decode(P, full, L, i, img, tx, ty);
+            decode(P, full, Lcur, i, img, tx, ty);
             const ImgDesc &D = P.imgs[img];
             Visit V;
             V.w = D.w;
             V.h = D.h;
-            V.lam = D.lam;
-            V.rule = P.rule | (D.adj << 2);  // F^- reading, operator, adjacency pair
             V.tw = P.tw;
             V.th = P.th;
-            V.H = H;
             V.Hs = Hs;
             V.hr = HR;
             V.g0 = g0;
-            V.start = P.start_phase;
             V.x0 = tx * P.tw;
             V.y0 = ty * P.th;
             const int u16 = D.dtype == THIN_U16;
             const int es = u16 ? 2 : 1;
-            V.pad = 16 / es;
-            const int bw = P.tw + 2 * V.pad;  // elements per shared row
-            const size_t pitch = D.pitch;
-            char *dst = reinterpret_cast<char *>(D.buf[src ^ 1]);
-            if (lane == 0) {
-                const uint32_t bytes = uint32_t(bw * es * (P.th + 2 * HR));
-                tma_load_2d(smem_u32(tile), &D.map[src], V.x0 - V.pad, V.y0 - HR, bar, bytes);
+            if (tid == 0) {
+                const int boxes = L.rows / L.box_rows;
+                const uint32_t box_bytes = uint32_t(L.box_rows) * uint32_t((P.tw + 2 * kPadCols) * es);
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(box_bytes * boxes)
+                             : "memory");
+                for (int b = 0; b < boxes; ++b)
+                    tma_load_2d(smem_u32(tile) + b * box_bytes, &D.map[src], V.x0 - kPadCols, V.y0 - HR + b * L.box_rows, bar);
+                ctrl->qn[0] = 0u;
+                ctrl->qn[1] = 0u;
+                ctrl->near = 0u;
+                ctrl->last = -1;
+                ctrl->next = gridDim.x + atomicAdd(&P.ctl->next_item[s % 3], 1u);
             }
-            // Stamps of the region (overlaps the load); the border ring never changes.  In shared
-            // memory a stamp is a byte, its distance from stamp0: 0 for anything before the last three
-            // phases (no phase of this step looks further back), 4 + j for phase j of the step.
-            const int stamp0 = int(g0 - P.start_phase) - 4;
+            // dirty bits of the tile and its halo (overlaps the load): a warp to a cell row, a lane to a cell
             {
-                const int32_t *gc = reinterpret_cast<const int32_t *>(D.cells);
-                const int cx0 = (V.x0 - V.pad) / 8 - 1, cy0 = (V.y0 - HR) / 2 - 1;
-                const int n = WL.ccols * WL.crows;
+                const unsigned char *bits = reinterpret_cast<const unsigned char *>(D.cells[src]);
+                const int gx = (V.x0 - kPadCols) / 8 + lane, gy0 = (V.y0 - HR) / 2;  // (both exact: multiples of 8 and 2)
+                const bool col = lane < (P.tw + 2 * kPadCols) / 8 && gx >= 0 && gx < D.cells_x;
 #pragma unroll 4
-                for (int e = lane; e < n; e += 32) {
-                    const int cy = div_small(e, WL.ccols, Mcc), cx = e - cy * WL.ccols;
-                    const int gx = cx0 + cx, gy = cy0 + cy;
-                    const bool ring = cx == 0 || cy == 0 || cx == WL.ccols - 1 || cy == WL.crows - 1;
-                    int age = 0;
-                    if (!ring && gx >= 0 && gy >= 0 && gx < D.cells_x && gy < D.cells_y)
-                        age = max(__ldcg(gc + size_t(gy) * D.cells_x + gx) - stamp0, 0);
-                    cells[e] = uint8_t(age);
+                for (int cr = warp; cr < words; cr += kWarps) {
+                    const int gy = gy0 + cr;
+                    unsigned v = 0;
+                    if (col && gy >= 0 && gy < D.cells_y) v = __ldcg(bits + size_t(gy) * D.cells_x + gx);
+                    const unsigned b0 = __ballot_sync(0xffffffffu, v & 1u), b1 = __ballot_sync(0xffffffffu, v & 2u);
+                    const unsigned b2 = __ballot_sync(0xffffffffu, v & 4u), b3 = __ballot_sync(0xffffffffu, v & 8u);
+                    if (lane < 4) dirty[lane * words + cr] = lane == 0 ? b0 : lane == 1 ? b1 : lane == 2 ? b2 : b3;
                 }
             }
             const bool ok = mbar_wait(bar, parity, P.timeout_ns);
-            parity ^= 1u;
-            if (!__all_sync(0xffffffffu, ok)) {
-                if (lane == 0) {
-                    atomicCAS(&P.ctl->error, 0, THIN_ERR_TIMEOUT);
-                    mbar_wait(bar, parity ^ 1u, P.timeout_ns);  // let the load in flight land (bounded)
-                }
+            if (!__syncthreads_and(ok)) {
+                mbar_wait(bar, parity, P.timeout_ns);  // let copies in flight land (bounded)
                 failed = true;
                 break;
             }
-            __syncwarp();
+            parity ^= 1u;
             int nlow = 0, chg_j = -1, ntest = 0;
-            if (u16)
-                visit_phases<uint16_t>(reinterpret_cast<uint16_t *>(tile), bw, cells, WL.ccols, queue, V, tabs, nlow,
-                                       chg_j, ntest);
-            else
-                visit_phases<uint8_t>(tile, bw, cells, WL.ccols, queue, V, tabs, nlow, chg_j, ntest);
-            tile_store(tile, bw * es, es, V, dst, pitch);
-            // stamps of the interior cells back to the image's stamp grid
+            const PointRule rule = point_rule(smem, P.rule | (D.adj << 2), D.lam, es, true);  // F^- reading, operator, pair
+            TileLayout Li = L;
+            Li.row_bytes = (P.tw + 2 * kPadCols) * es;
+            if (u16) visit_phases<uint16_t>(Li, smem, V, rule, nlow, ntest, chg_j);
+            else visit_phases<uint8_t>(Li, smem, V, rule, nlow, ntest, chg_j);
+            tile_store(tile, Li.row_bytes, es, V, reinterpret_cast<char *>(D.buf[src ^ 1]), D.pitch);
+            // the tile's dirty bits, and which neighbours they can reach in the next step
             {
-                int32_t *gc = reinterpret_cast<int32_t *>(D.cells);
-                const int icx = V.tw / 8, icy = V.th / 2;
-                const int cxa = V.x0 / 8, cya = V.y0 / 2;
-                const int ox = V.pad / 8 + 1, oy = HR / 2 + 1;
-                const uint32_t Mi = div_magic(icx);
-#pragma unroll 4
-                for (int e = lane; e < icx * icy; e += 32) {
-                    const int cy = div_small(e, icx, Mi), cx = e - cy * icx;
-                    const int gx = cxa + cx, gy = cya + cy;
-                    if (gx < D.cells_x && gy < D.cells_y)
-                        __stcg(gc + size_t(gy) * D.cells_x + gx, stamp0 + cells[(oy + cy) * WL.ccols + ox + cx]);
+                unsigned char *bits = reinterpret_cast<unsigned char *>(D.cells[src ^ 1]);
+                const int gx = V.x0 / 8 + lane, gy0 = V.y0 / 2;
+                const int cols = P.tw / 8, rows = P.th / 2;
+                const int zx = (H + 2 + 7) / 8, zy = (H + 2 + 1) / 2;  // cells within reach of an edge
+                const unsigned left = 0xffffffffu >> (32 - min(zx, 32)), right = left << max(cols - zx, 0);
+                unsigned near = 0;
+                for (int cr = warp; cr < rows; cr += kWarps) {
+                    const int gy = gy0 + cr;
+                    const uint32_t *w = dirty + HR / 2 + cr;
+                    const int b = lane + kPadCols / 8;
+                    unsigned v = 0;
+                    if (lane < cols && gx < D.cells_x && gy < D.cells_y) {
+                        v = ((w[0] >> b) & 1u) | (((w[words] >> b) & 1u) << 1) | (((w[2 * words] >> b) & 1u) << 2) |
+                            (((w[3 * words] >> b) & 1u) << 3);
+                        __stcg(bits + size_t(gy) * D.cells_x + gx, static_cast<unsigned char>(v));
+                    }
+                    const unsigned any = __ballot_sync(0xffffffffu, v != 0);
+                    const unsigned xs = (any & left ? 1u : 0u) | (any ? 2u : 0u) | (any & right ? 4u : 0u);
+                    near |= (xs << 3) | (cr < zy ? xs : 0u) | (cr >= rows - zy ? xs << 6 : 0u);
                 }
+                if (lane == 0 && near) atomicOr(&ctrl->near, near);
             }
             nlow = __reduce_add_sync(0xffffffffu, nlow);
             ntest = __reduce_add_sync(0xffffffffu, ntest);
             const int maxj = __reduce_max_sync(0xffffffffu, chg_j);
-            // order this warp's generic shared and global writes before later TMA traffic
+            if (lane == 0) {
+                if (maxj >= 0) atomicMax(&ctrl->last, maxj);
+                if (nlow) atomicAdd(&P.st[img].lowered, (unsigned long long)nlow);
+                if (ntest) atomicAdd(&P.st[img].tested, (unsigned long long)ntest);
+            }
+            // order this block's generic shared and global writes before later TMA traffic
             asm volatile("fence.proxy.async;" ::: "memory");
-            __syncwarp();
-            if (lane < 9 && maxj >= 0) {
-                const int dx = lane % 3 - 1, dy = lane / 3 - 1;
-                const bool self = dx == 0 && dy == 0;
-                const bool late = maxj >= Hs - 3;
-                const int ntx = tx + dx, nty = ty + dy;
-                if ((self || late) && ntx >= 0 && ntx < D.tiles_x && nty >= 0 && nty < D.tiles_y) {
+            __syncthreads();
+            i = ctrl->next;
+            if (tid < 9) {
+                const int dx = tid % 3 - 1, dy = tid / 3 - 1;
+                const int ntx = tx + dx, nty = ty + dy, last = ctrl->last;
+                const bool list = ((ctrl->near >> tid) & 1u) || (tid == 4 && last >= 0);
+                if (list && ntx >= 0 && ntx < D.tiles_x && nty >= 0 && nty < D.tiles_y) {
                     const int gt = D.tile_base + nty * D.tiles_x + ntx;
                     if (atomicMax(&P.listed[gt], s + 1) < s + 1) {
                         const unsigned pos = atomicAdd(&P.ctl->list_count[(s + 1) % 3], 1u);
@@ -497,20 +490,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
                         atomicMax(&P.st[img].last_listed, s + 1);
                     }
                 }
+                if (tid == 4) {
+                    if (last >= 0) atomicMax(&P.st[img].last_change, g0 + last);
+                    atomicAdd(&P.st[img].tiles_visited, 1ull);
+                    atomicMax(&P.st[img].last_step, s);
+                }
             }
-            if (lane == 0) {
-                if (nlow) atomicAdd(&P.st[img].lowered, (unsigned long long)nlow);
-                if (maxj >= 0) atomicMax(&P.st[img].last_change, g0 + maxj);
-                atomicAdd(&P.st[img].tiles_visited, 1ull);
-                atomicAdd(&P.st[img].tested, (unsigned long long)ntest);
-                atomicMax(&P.st[img].last_step, s);
-            }
-            unsigned nxt = 0;
-            if (lane == 0) nxt = nwarps + atomicAdd(&P.ctl->next_item[s % 3], 1u);
-            i = __shfl_sync(0xffffffffu, nxt, 0);
+            __syncthreads();  // the control words are read before the next visit sets them
         }
         if (__syncthreads_or(failed)) {
-            if (threadIdx.x == 0) atomicCAS(&P.ctl->error, 0, THIN_ERR_TIMEOUT);
+            if (tid == 0) atomicCAS(&P.ctl->error, 0, THIN_ERR_TIMEOUT);
             return;
         }
         const bool skip = P.debug == 1 && blockIdx.x == 0 && s == 0;
@@ -518,9 +507,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
         g0 += Hs;
         const long long ran = g0 - P.start_phase;
         const unsigned next = *reinterpret_cast<volatile unsigned *>(&P.ctl->list_count[(s + 1) % 3]);
-        const bool stop = (P.max_phases >= 0 && ran >= P.max_phases) || (ran > 3 && next == 0);
+        const bool stop = (P.max_phases >= 0 && ran >= P.max_phases) || next == 0;
         if (stop) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) P.ctl->steps = s + 1;
+            if (blockIdx.x == 0 && tid == 0) P.ctl->steps = s + 1;
             return;
         }
     }
@@ -567,27 +556,78 @@ EncodeTiledFn encode_fn()
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Shared-memory layout of one warp for tiles tw x th and halo rows hr.  The
-// tile buffer fits the widest element present; the stamp grid and the queue
-// fit u8 geometry (16 pad elements either side), which is the wider in cells.
-WarpLayout warp_layout(int tw, int th, int hr, bool any16)
+// Shared memory of a block for tiles tw x th with hr halo rows.  A tile of more
+// than 256 staged rows takes two TMA boxes, each starting at a multiple of 128 bytes.
+TileLayout tile_layout(int tw, int th, int hr, bool any16)
 {
-    WarpLayout L;
-    const int bw_bytes = any16 ? (tw + 16) * 2 : tw + 32;
-    const int cols8 = (tw + 32) / 8;  // cells per shared row of a u8 tile (u16: fewer)
-    const int rows = th + 2 * hr;
-    L.tile_bytes = int(align_up(size_t(bw_bytes) * rows + 16, 16));
-    L.ccols = cols8 + 2;
-    L.crows = rows / 2 + 2;
-    L.cell_off = L.tile_bytes;
-    const int max_items = (rows / 2 + 1) * (cols8 + 1);
-    L.queue_off = int(align_up(size_t(L.cell_off) + size_t(L.ccols) * L.crows, 16));
-    L.bar_off = int(align_up(size_t(L.queue_off) + 2 * size_t(max_items), 16));
-    L.bytes = int(align_up(size_t(L.bar_off) + 16, 128));
+    TileLayout L;
+    L.row_bytes = (tw + 2 * kPadCols) * (any16 ? 2 : 1);
+    L.rows = th + 2 * hr;
+    L.box_rows = L.rows;
+    if (L.rows > 256) {
+        L.box_rows = int(align_up(size_t(L.rows + 1) / 2, 8));
+        L.rows = 2 * L.box_rows;
+    }
+    L.dirty_off = int(align_up(size_t(kOffTile) + size_t(L.row_bytes) * L.rows + 16, 16));
+    L.queue_off = L.dirty_off + 4 * 4 * (L.rows / 2);
+    L.bytes = L.queue_off + 2 * 32 * (L.rows / 2);
     return L;
 }
 
+// Halo rows for steps of H phases: one pixel more than phases, even.
+int halo_rows(int H) { return (H + 2) / 2 * 2; }
+
+// Tile shape and phases per step.  What the caller set is taken as it is (and
+// checked); with nothing set the largest of these shapes that still gives every
+// SM two tiles: a large tile has less halo (224 x 152 with rings of 1 to 15:
+// 17 % more points; 64 x 32 with 1 to 8: 46 %), and two blocks of 113 KB share an
+// SM.  Steps of 6 / 8 / 12 / 15 phases: 8192^2 u16 at lambda = 0 4.83 / 4.65 /
+// 4.77 / 4.75 ms, at lambda = 30 15.1 / 14.3 / 14.0 / 13.9 ms, the served
+// requests 72.7 / 70.5 / 60.8 / 59.3 ms; one block of 16 warps an SM, with
+// tiles twice as high: 4.68, 13.9 and 55 ms against 58.9; three of 5 warps:
+// 5.6, 15.8 and 73 ms.
+int tiled_shape(const JobSpec *jobs, int n, bool any16, const thin_options &opt, int *tw, int *th, int *H)
+{
+    if (opt.tile_w || opt.tile_h || opt.halo) {
+        tiled_defaults(any16 ? THIN_U16 : THIN_U8, tw, th, H);
+        if (opt.tile_w) *tw = opt.tile_w;
+        if (opt.tile_h) *th = opt.tile_h;
+        if (opt.halo) *H = opt.halo;
+        const int max_halo = any16 ? 8 : 16;
+        if (*H < kMinHalo || *H > max_halo || *tw < 16 || *tw > 224 || *tw % 16 || *th < 8 || *th % 2 ||
+            std::min(*tw, *th) < *H + 1 || *th + 2 * (*H + (*H & 1)) > 256)
+            return THIN_ERR_ARG;
+        *H = std::min(*H, kMaxStep);
+        return THIN_OK;
+    }
+    static const int shapes[2][5][3] = {{{224, 304, 15}, {224, 160, 15}, {224, 80, 8}, {128, 64, 8}, {64, 32, 8}},
+                                        {{224, 152, 15}, {224, 96, 15}, {128, 96, 8}, {96, 48, 8}, {64, 32, 8}}};
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    for (const auto &s : shapes[any16 ? 1 : 0]) {
+        *tw = s[0];
+        *th = s[1];
+        *H = s[2];
+        size_t tiles = 0;
+        for (int k = 0; k < n; ++k)
+            tiles += size_t((jobs[k].w + *tw - 1) / *tw) * size_t((jobs[k].h + *th - 1) / *th);
+        if (tiles >= size_t(2 * sms)) break;
+    }
+    return THIN_OK;
+}
+
 }  // namespace
+
+bool tiled_fills(const JobSpec *jobs, int n, int *tw, int *th, int *H)
+{
+    bool any16 = false;
+    for (int k = 0; k < n; ++k) any16 |= jobs[k].dtype == THIN_U16;
+    thin_options o;
+    std::memset(&o, 0, sizeof o);
+    tiled_shape(jobs, n, any16, o, tw, th, H);
+    return *H == kMaxStep;  // (the large shapes)
+}
 
 void tiled_defaults(int dtype, int *tw, int *th, int *halo)
 {
@@ -615,20 +655,11 @@ int tiled_prepare(const JobSpec *jobs, int n, const thin_options &opt, cudaStrea
     *out = nullptr;
     bool any16 = false;
     for (int k = 0; k < n; ++k) any16 |= jobs[k].dtype == THIN_U16;
-    int tw = opt.tile_w, th = opt.tile_h, H = opt.halo;
-    {
-        int dw, dh, dH;
-        tiled_defaults(any16 ? THIN_U16 : THIN_U8, &dw, &dh, &dH);
-        if (!tw) tw = dw;
-        if (!th) th = dh;
-        if (!H) H = dH;
-    }
-    const int max_halo = any16 ? 8 : 16;  // the 16-byte left pad holds the halo columns
-    if (H < kMinHalo || H > max_halo || tw < 16 || tw > 224 || tw % 16 || th < 8 || th % 2 ||
-        std::min(tw, th) < H + 1)
-        return THIN_ERR_ARG;
-    const int HR = H + (H & 1);
-    if (th + 2 * HR > 256) return THIN_ERR_ARG;
+    int tw, th, H;
+    const int shape_rc = tiled_shape(jobs, n, any16, opt, &tw, &th, &H);
+    if (shape_rc != THIN_OK) return shape_rc;
+    const int HR = halo_rows(H);
+    const TileLayout TL = tile_layout(tw, th, HR, any16);
     EncodeTiledFn enc = encode_fn();
     if (!enc) return THIN_ERR_CUDA;
 
@@ -644,7 +675,7 @@ int tiled_prepare(const JobSpec *jobs, int n, const thin_options &opt, cudaStrea
     // ---- layout of one scratch allocation
     std::vector<ImgDesc> &descs = T->descs;
     descs.resize(n);
-    std::vector<size_t> buf_off(n), cpy_off(n), cell_off(n);
+    std::vector<size_t> buf_off(n), cpy_off(n), cell_off(n), cell1_off(n);
     size_t off = 0;
     const size_t o_desc = off;
     off = align_up(off + sizeof(ImgDesc) * n, 256);
@@ -689,9 +720,13 @@ int tiled_prepare(const JobSpec *jobs, int n, const thin_options &opt, cudaStrea
     T->o_cells = off;
     for (int k = 0; k < n; ++k) {
         cell_off[k] = off;
-        off = align_up(off + sizeof(int32_t) * size_t(descs[k].cells_x) * descs[k].cells_y, 256);
+        off = align_up(off + size_t(descs[k].cells_x) * descs[k].cells_y, 256);
     }
     T->cells_bytes = off - T->o_cells;
+    for (int k = 0; k < n; ++k) {  // (written by the first step, which visits every tile)
+        cell1_off[k] = off;
+        off = align_up(off + size_t(descs[k].cells_x) * descs[k].cells_y, 256);
+    }
     T->o_listed = off;
     off = align_up(off + sizeof(int) * total_tiles, 256);
     const size_t o_lists = off;
@@ -715,11 +750,11 @@ int tiled_prepare(const JobSpec *jobs, int n, const thin_options &opt, cudaStrea
         void *b1 = base + buf_off[k];
         D.buf[0] = reinterpret_cast<unsigned long long>(b0);
         D.buf[1] = reinterpret_cast<unsigned long long>(b1);
-        D.cells = reinterpret_cast<unsigned long long>(base + cell_off[k]);
-        const int pad = J.dtype == THIN_U16 ? 8 : 16;
+        D.cells[0] = reinterpret_cast<unsigned long long>(base + cell_off[k]);
+        D.cells[1] = reinterpret_cast<unsigned long long>(base + cell1_off[k]);
         const cuuint64_t gdim[2] = {cuuint64_t(J.w), cuuint64_t(J.h)};
         const cuuint64_t gstr[1] = {cuuint64_t(D.pitch)};
-        const cuuint32_t box[2] = {cuuint32_t(tw + 2 * pad), cuuint32_t(th + 2 * HR)};
+        const cuuint32_t box[2] = {cuuint32_t(tw + 2 * kPadCols), cuuint32_t(TL.box_rows)};
         const cuuint32_t est[2] = {1, 1};
         for (int q = 0; q < 2; ++q) {
             void *bp = q ? b1 : b0;
@@ -766,8 +801,8 @@ int tiled_prepare(const JobSpec *jobs, int n, const thin_options &opt, cudaStrea
     P.timeout_ns = 2000000000ull;
     if (const char *t = std::getenv("THIN_TIMEOUT_NS")) P.timeout_ns = std::strtoull(t, nullptr, 10);
     P.debug = opt.reserved;
-    P.wl = warp_layout(tw, th, HR, any16);
-    T->smem = 128 + kSmemTabs + kWarps * P.wl.bytes;
+    P.tl = TL;
+    T->smem = 128 + TL.bytes;
     {
         int optin = 0;
         cudaFuncAttributes fa;
@@ -783,7 +818,7 @@ int tiled_prepare(const JobSpec *jobs, int n, const thin_options &opt, cudaStrea
     int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_engine, kThreads, T->smem);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
-    T->grid = std::max(1, std::min(sms * per_sm, (total_tiles + kWarps - 1) / kWarps));
+    T->grid = std::max(1, std::min(sms * per_sm, total_tiles));
     if (max_grid > 0) T->grid = std::min(T->grid, max_grid);
     if (opt.reserved == 1) T->grid = std::max(T->grid, std::min(2, sms * per_sm));
     if (e != cudaSuccess) {
@@ -811,7 +846,7 @@ cudaError_t tiled_enqueue(const TiledPrepared *T, cudaStream_t stream)
         e = cudaMemcpyAsync(base + T->o_stat, base + T->o_stat0, sizeof(ImgStat) * T->n, cudaMemcpyDeviceToDevice, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + T->o_ctl, base + T->o_ctl0, sizeof(Ctl), cudaMemcpyDeviceToDevice, stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(base + T->o_listed, 0xff, sizeof(int) * T->total_tiles, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + T->o_cells, 0, T->cells_bytes, stream);  // every cell: changed at the first phase
+    if (e == cudaSuccess) e = cudaMemsetAsync(base + T->o_cells, 0x0f, T->cells_bytes, stream);  // every group dirty
     if (e == cudaSuccess) {
         void *args[] = {const_cast<EngineArgs *>(&T->P)};
         e = cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_engine), dim3(T->grid), dim3(kThreads), args, T->smem,
@@ -978,20 +1013,11 @@ int tiled_run_noalloc(const JobSpec &J, const thin_options &opt, cudaStream_t st
         return THIN_ERR_NOT_CONVERGED;
     }
     const bool is16 = J.dtype == THIN_U16;
-    int tw = opt.tile_w, th = opt.tile_h, H = opt.halo;
-    {
-        int dw, dh, dH;
-        tiled_defaults(J.dtype, &dw, &dh, &dH);
-        if (!tw) tw = dw;
-        if (!th) th = dh;
-        if (!H) H = dH;
-    }
-    const int max_halo = is16 ? 8 : 16;
-    if (H < kMinHalo || H > max_halo || tw < 16 || tw > 224 || tw % 16 || th < 8 || th % 2 ||
-        std::min(tw, th) < H + 1)
-        return THIN_ERR_ARG;
-    const int HR = H + (H & 1);
-    if (th + 2 * HR > 256) return THIN_ERR_ARG;
+    int tw, th, H;
+    const int shape_rc = tiled_shape(&J, 1, is16, opt, &tw, &th, &H);
+    if (shape_rc != THIN_OK) return shape_rc;
+    const int HR = halo_rows(H);
+    const TileLayout TL = tile_layout(tw, th, HR, is16);
     EncodeTiledFn enc = encode_fn();
     if (!enc) return THIN_ERR_CUDA;
 
@@ -1028,7 +1054,9 @@ int tiled_run_noalloc(const JobSpec &J, const thin_options &opt, cudaStream_t st
     const size_t o_cpy = off;
     if (D.copy_in) off = align_up(off + D.pitch * J.h, 256);
     const size_t o_cells = off;
-    const size_t cells_bytes = sizeof(int32_t) * size_t(D.cells_x) * D.cells_y;
+    const size_t cells_bytes = size_t(D.cells_x) * D.cells_y;
+    off = align_up(off + cells_bytes, 256);
+    const size_t o_cells1 = off;
     off = align_up(off + cells_bytes, 256);
     const size_t o_listed = off;
     off = align_up(off + sizeof(int) * total_tiles, 256);
@@ -1046,12 +1074,12 @@ int tiled_run_noalloc(const JobSpec &J, const thin_options &opt, cudaStream_t st
         e = cudaMemcpy2DAsync(b0, D.pitch, J.img, J.pitch, size_t(J.w) * es, J.h, cudaMemcpyDeviceToDevice, stream);
     D.buf[0] = reinterpret_cast<unsigned long long>(b0);
     D.buf[1] = reinterpret_cast<unsigned long long>(b1);
-    D.cells = reinterpret_cast<unsigned long long>(base + o_cells);
+    D.cells[0] = reinterpret_cast<unsigned long long>(base + o_cells);
+    D.cells[1] = reinterpret_cast<unsigned long long>(base + o_cells1);
     {
-        const int pad = is16 ? 8 : 16;
         const cuuint64_t gdim[2] = {cuuint64_t(J.w), cuuint64_t(J.h)};
         const cuuint64_t gstr[1] = {cuuint64_t(D.pitch)};
-        const cuuint32_t box[2] = {cuuint32_t(tw + 2 * pad), cuuint32_t(th + 2 * HR)};
+        const cuuint32_t box[2] = {cuuint32_t(tw + 2 * kPadCols), cuuint32_t(TL.box_rows)};
         const cuuint32_t est[2] = {1, 1};
         for (int q = 0; q < 2; ++q) {
             CUresult r = enc(&D.map[q], is16 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 2,
@@ -1075,7 +1103,7 @@ int tiled_run_noalloc(const JobSpec &J, const thin_options &opt, cudaStream_t st
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_stat, &st0, sizeof st0, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_ctl, &ctl0, sizeof ctl0, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(base + o_listed, 0xff, sizeof(int) * total_tiles, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + o_cells, 0, cells_bytes, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(base + o_cells, 0x0f, cells_bytes, stream);
 
     EngineArgs P;
     std::memset(&P, 0, sizeof P);
@@ -1096,8 +1124,8 @@ int tiled_run_noalloc(const JobSpec &J, const thin_options &opt, cudaStream_t st
     P.timeout_ns = 2000000000ull;
     if (const char *t = std::getenv("THIN_TIMEOUT_NS")) P.timeout_ns = std::strtoull(t, nullptr, 10);
     P.debug = 0;
-    P.wl = warp_layout(tw, th, HR, is16);
-    const int smem = 128 + kSmemTabs + kWarps * P.wl.bytes;
+    P.tl = TL;
+    const int smem = 128 + TL.bytes;
 
     int dev = 0, sms = 0, per_sm = 0, optin = 0;
     cudaFuncAttributes fa;
@@ -1109,7 +1137,7 @@ int tiled_run_noalloc(const JobSpec &J, const thin_options &opt, cudaStream_t st
     if (e == cudaSuccess) e = allow_max_dynamic_smem(reinterpret_cast<const void *>(k_engine));
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_engine, kThreads, smem);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
-    const int grid = std::max(1, std::min(sms * per_sm, (total_tiles + kWarps - 1) / kWarps));
+    const int grid = std::max(1, std::min(sms * per_sm, total_tiles));
     if (e == cudaSuccess) {
         void *args[] = {&P};
         e = cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_engine), dim3(grid), dim3(kThreads), args, smem,

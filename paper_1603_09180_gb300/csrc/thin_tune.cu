@@ -14,12 +14,11 @@ struct Candidate {
     int tw, th, halo;
 };
 
-// Tile shapes and halo depths the tiled engine accepts for both dtypes
-// (tile width a multiple of 16 up to 224, even height, halo <= 8 and below
-// the shorter tile side, tile height + 2 halo rows <= 256).
+// Tile shapes and phases per step (thin_tiled.cu: tiled_shape): large tiles
+// have less halo, small ones give a lone image enough tiles for every SM.
 const Candidate kCandidates[] = {
-    {64, 32, 8}, {64, 32, 6}, {64, 32, 4}, {128, 32, 8}, {64, 64, 8}, {128, 64, 8},
-    {32, 32, 8}, {96, 48, 8}, {128, 16, 8}, {224, 32, 8}, {48, 64, 8}, {64, 16, 6},
+    {224, 240, 8}, {224, 160, 8}, {224, 96, 8}, {160, 96, 8}, {128, 128, 8}, {128, 64, 8},
+    {96, 96, 8}, {96, 48, 8}, {64, 64, 8}, {64, 32, 8}, {128, 64, 6}, {64, 32, 6},
 };
 
 }  // namespace

@@ -1,0 +1,30 @@
+"""The tiled engine's tiles at their edges, against the oracle: the smallest tile, tiles of one and of two
+TMA boxes, the longest steps, images that end inside, at and just past a tile, caps and resumes inside a step."""
+import numpy as np
+import pytest
+
+pytest.importorskip("torch")
+import torch  # noqa: E402
+
+import oracle  # noqa: E402
+from paper_1603_09180_gb300 import synth, thin  # noqa: E402
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")]
+
+
+@pytest.mark.parametrize("tile,halo", [(None, 0), ((16, 8), 3), ((32, 18), 16), ((224, 240), 8), ((208, 240), 7)])
+@pytest.mark.parametrize("h,w,dtype,lam", [(241, 225, "u8", 7), (240, 224, "u8", 0), (97, 241, "u16", 90), (9, 17, "u8", 5)])
+def test_tiles(h, w, dtype, lam, tile, halo):
+    if dtype == "u16" and halo > 8:
+        pytest.skip("u16 takes steps of at most 8 phases")
+    img = synth.value_noise_image(h, w, dtype, seed=h + 5 * w)
+    ref, rst = oracle.thin(img, lam)
+    t = torch.from_numpy(img).cuda()
+    st = thin.run(t, lam, kernel="tiled", tile=tile, halo=halo)
+    assert np.array_equal(t.cpu().numpy(), ref)
+    assert st["converged"] == 1 and st["lowered"] == rst["lowered"] and st["last_change_phase"] == rst["last_change_phase"]
+    t = torch.from_numpy(img).cuda()
+    at = 0
+    for cap in (1, 2, 9, -1):
+        at = thin.run(t, lam, kernel="tiled", tile=tile, halo=halo, start_phase=at, max_phases=cap)["end_phase"]
+    assert np.array_equal(t.cpu().numpy(), ref)
