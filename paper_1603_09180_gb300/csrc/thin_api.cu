@@ -78,6 +78,26 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
         for (int k = 0; k < n; ++k)
             cls[k] = resident_cluster_size(specs[k].w, specs[k].h, specs[k].dtype, limit, nullptr, nullptr);
     }
+    // Many images that need clusters of 16 or 8 go to the tiled engine too: few
+    // such clusters fit on the GPU at once (they lie within a GPC), so they run in
+    // waves, while tiles of all the images fill every SM.  Resident against tiled:
+    // 8 / 24 / 64 u8 images of 1400^2 (16 blocks) at lambda = 20 25.8 / 58.3 /
+    // 154.7 ms against 28.1 / 52.0 / 104.9; u16 of 1000^2 at lambda = 80
+    // 13.1 / 32.7 / 83.5 against 16.4 / 25.8 / 49.5; u8 of 1000^2 (8 blocks)
+    // 14.0 / 23.0 / 56.2 against 16.6 / 30.2 / 52.1, and better together with
+    // larger images: 1024 uneven images with clusters up to 16 / 8 / 4 kept
+    // resident 262 / 221 / 202 ms.  (Serving, which passes allow_wide = false,
+    // keeps them resident: its small lanes retire image by image.  So does a call
+    // that sets a tile shape, which not every image may take.)
+    if (allow_wide && o.kernel == THIN_KERNEL_AUTO && !o.tile_w && !o.tile_h && !o.halo) {
+        int count[17] = {};
+        for (int k = 0; k < n; ++k) ++count[cls[k]];
+        const int huge = count[0] > kWideMax ? count[0] : 0;
+        const bool tile16 = count[16] + huge >= 24;
+        const bool tile8 = count[8] >= 64 || ((tile16 || huge >= 24) && count[8] >= 32);
+        for (int k = 0; k < n; ++k)
+            if ((cls[k] == 16 && tile16) || (cls[k] == 8 && tile8)) cls[k] = -1;
+    }
     int eligible = 0, sms = 0, dev = 0;
     for (int k = 0; k < n; ++k) eligible += cls[k] > 0;
     cudaGetDevice(&dev);
@@ -110,7 +130,7 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     for (int k = 0; k < n; ++k) nwide += cls[k] == 0 && strips[k] > 0;
     const bool use_wide = nwide > 0 && (nwide <= kWideMax || o.kernel == THIN_KERNEL_RESIDENT);
     for (int k = 0; k < n; ++k) {
-        if (cls[k] != 0) continue;
+        if (cls[k] > 0) continue;
         if (use_wide && strips[k] > 0) G->wide.push_back({k, strips[k], csize[k]});
         else G->tiled.push_back(k);
     }

@@ -28,3 +28,20 @@ def test_tiles(h, w, dtype, lam, tile, halo):
     for cap in (1, 2, 9, -1):
         at = thin.run(t, lam, kernel="tiled", tile=tile, halo=halo, start_phase=at, max_phases=cap)["end_phase"]
     assert np.array_equal(t.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("n", [23, 24])
+def test_many_cluster16_images_go_to_tiles(n):
+    """24 images that need a cluster of 16 blocks go to the tiled engine, 23 do not; the result is the same."""
+    imgs = [synth.value_noise_image(1300, 1310, "u8", seed=s) for s in (1, 2)]
+    want = []
+    for im in imgs:
+        t = torch.from_numpy(im).cuda()
+        thin.run(t, 3, kernel="resident")
+        want.append(t)
+    work = [torch.from_numpy(imgs[k % 2]).cuda() for k in range(n)]
+    stats, rc = thin.batch(work, [3] * n)
+    assert rc == 0
+    assert all((s["tiles_visited"] > 0) == (n >= 24) for s in stats)
+    for k, t in enumerate(work):
+        assert torch.equal(t, want[k % 2])
