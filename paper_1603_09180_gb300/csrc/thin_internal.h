@@ -183,6 +183,26 @@ bool tiled_fills(const JobSpec *jobs, int n, int *tw, int *th, int *H);
 // where the caller sets only some of them.
 void tiled_defaults(int dtype, int *tw, int *th, int *halo);
 
+// Mosaic engine (thin_mosaic.cu): a few images whose tiles all fit in shared
+// memory at once, one block to a tile.
+struct MosaicShape {
+    int tw, th, halo;  // tile, phases per step
+};
+// The best tile shape for these images; false if they do not fit.
+bool mosaic_shape(const JobSpec *jobs, int n, MosaicShape *out);
+struct MosaicPrepared {
+    int n = 0, es = 1, grid = 0, smem = 0, halo = 0;
+    bool async_alloc = true;
+    char *base = nullptr, *live = nullptr;  // one allocation; the part to zero before a run
+    size_t live_bytes = 0, o_st = 0, o_err = 0;
+    std::vector<char> args;                 // the kernel's argument block
+};
+int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const thin_options &opt, cudaStream_t stream,
+                   bool async_alloc, MosaicPrepared *M);
+cudaError_t mosaic_enqueue(const MosaicPrepared &M, cudaStream_t stream);
+int mosaic_collect(const MosaicPrepared &M, const thin_options &opt, cudaStream_t stream, thin_stats *out);
+void mosaic_release(MosaicPrepared &M, cudaStream_t stream);
+
 int cuda_status(cudaError_t e);
 
 // Resident launch groups of a batch at most: one per cluster size (1, 2, 4,
@@ -198,6 +218,8 @@ struct Grouping {
         int job, strips, C;
     };
     std::vector<Wide> wide;  // one wide launch each
+    std::vector<int> mosaic;  // one launch
+    MosaicShape mosaic_tile;
     std::vector<int> tiled;
 };
 // allow_wide: large images may take the wide resident mode (a cooperative
@@ -218,6 +240,8 @@ struct Execution {
     std::vector<std::vector<int>> res_idx;
     std::vector<ResidentPrepared> wide;
     std::vector<int> wide_idx;
+    MosaicPrepared mosaic;
+    std::vector<int> mosaic_idx;
     TiledPrepared *tiled = nullptr;
     std::vector<int> tiled_idx;
     int prepare(const std::vector<JobSpec> &specs, const Grouping &G, const thin_options &o, cudaStream_t s,

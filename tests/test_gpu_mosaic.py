@@ -1,0 +1,51 @@
+"""The mosaic engine (a few images, a block to a tile, rims exchanged through flags) against the oracle.
+
+Sizes with one tile, tiles that end at, inside and one pixel past the image, rows that do not start at
+16-byte boundaries; caps and resumes inside a step; 16 images (the most that take it) and 17."""
+import numpy as np
+import pytest
+
+pytest.importorskip("torch")
+import torch  # noqa: E402
+
+import oracle  # noqa: E402
+from paper_1603_09180_gb300 import synth, thin  # noqa: E402
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")]
+
+
+@pytest.mark.parametrize("h,w,dtype,lam,op,adj", [
+    (3, 3, "u8", 4, "thinning", 0), (16, 32, "u8", 0, "thinning", 0), (17, 33, "u16", 60, "thinning", 0),
+    (128, 256, "u8", 12, "thinning", 0), (129, 257, "u8", 12, "skeleton", 0), (33, 700, "u16", 200, "thinning", 1),
+    (600, 35, "u8", 0, "skeleton", 1)])
+def test_mosaic(h, w, dtype, lam, op, adj):
+    img = synth.value_noise_image(h, w, dtype, seed=2 * h + w)
+    ref, rst = oracle.thin(img, lam, op={"thinning": 0, "skeleton": 1}[op], adj=adj)
+    base = torch.from_numpy(img).cuda()
+    for pad, at in ((0, 0), (5, 3)):  # packed rows, then rows at odd addresses
+        t = torch.empty((h, w + pad), dtype=base.dtype, device="cuda")[:, at:at + w]
+        t.copy_(base)
+        st = thin.run(t, lam, op=op, adj=adj)
+        assert np.array_equal(t.cpu().numpy(), ref)
+        assert st["converged"] == 1 and st["lowered"] == rst["lowered"] and st["last_change_phase"] == rst["last_change_phase"]
+    t = base.clone()
+    g, low = 0, 0
+    for cap in (1, 2, 14, 15, 16, -1):
+        st = thin.run(t, lam, op=op, adj=adj, start_phase=g, max_phases=cap)
+        assert cap < 0 or st["phases"] <= cap
+        g, low = st["end_phase"], low + st["lowered"]
+    assert np.array_equal(t.cpu().numpy(), ref) and low == rst["lowered"]
+
+
+@pytest.mark.parametrize("n", [2, 16, 17])
+def test_few_images(n):
+    shapes = [(40 + 17 * k, 90 + 11 * k) for k in range(n)]
+    imgs = [synth.value_noise_image(h, w, "u8", seed=h) for h, w in shapes]
+    lams = [(0, 6, 15)[k % 3] for k in range(n)]
+    work = [torch.from_numpy(a).cuda() for a in imgs]
+    stats, rc = thin.batch(work, lams)
+    assert rc == 0
+    for a, lam, t, st in zip(imgs, lams, work, stats):
+        ref, rst = oracle.thin(a, lam)
+        assert np.array_equal(t.cpu().numpy(), ref)
+        assert st["lowered"] == rst["lowered"] and st["last_change_phase"] == rst["last_change_phase"]
