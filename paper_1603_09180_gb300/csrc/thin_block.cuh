@@ -89,8 +89,9 @@ __device__ __forceinline__ bool work_queue(const PieceMap &m, const PointRule &r
     // u8 batch lost 3 %.
     constexpr int kLaneItems = THREADS / 4;
     bool moved = false;
-    if (N <= kLaneItems) {
-        const int k = int(threadIdx.x) >> 2, j4 = threadIdx.x & 3;
+    const int rest = N % THREADS, quads = rest <= kLaneItems ? N - rest : N;
+    if (quads < N) {
+        const int k = quads + (int(threadIdx.x) >> 2), j4 = threadIdx.x & 3;
         if (k < N) {
             const int code = queue[k];
             const int cr = code >> m.cbits, cc = code - (cr << m.cbits);
@@ -109,8 +110,9 @@ __device__ __forceinline__ bool work_queue(const PieceMap &m, const PointRule &r
                 if (A) mark_neighbours(m, cr, cc, A << (8 * j4), px, py);
             }
         }
-    } else {
-        for (int k = threadIdx.x; k < N; k += THREADS) {
+    }
+    {
+        for (int k = threadIdx.x; k < quads; k += THREADS) {
             const int code = queue[k];
             const int cr = code >> m.cbits, cc = code - (cr << m.cbits);
             const int first = (lo - px - 8 * cc + 1) >> 1, last = (hi - px - 8 * cc) >> 1;  // of the points 0 .. 3
