@@ -117,13 +117,14 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     int spread = 1;
     while (eligible > 0 && spread < 8 && spread * 2 * eligible <= sms) spread *= 2;
     // one launch per cluster size and element size (the kernel is built for each element size)
-    for (int C = 1; C <= 16; C *= 2)
+    for (int C : kClusterSizes)
         for (int dt = THIN_U8; dt <= THIN_U16; ++dt) {
             std::vector<int> idx;
             for (int k = 0; k < n; ++k) {
                 if (cls[k] <= 0 || specs[k].dtype != dt) continue;
                 int c = cls[k];
-                while (c < spread && specs[k].h / (2 * c) >= 32) c *= 2;
+                for (int wider : kClusterSizes)
+                    if (wider > c && wider <= spread && specs[k].h / wider >= 32) c = wider;
                 if (c == C) idx.push_back(k);
             }
             if (!idx.empty()) G->resident.push_back({C, idx});

@@ -48,7 +48,7 @@ int naive_run(const JobSpec &job, const thin_options &opt, cudaStream_t stream, 
 int tiled_run(const JobSpec *jobs, int n, const thin_options &opt, cudaStream_t stream, thin_stats *out);
 
 // Resident engine: each image held in the shared memory of one thread-block
-// cluster of C blocks (1, 2, 4 or 8) of 16 warps, one block per SM, for its
+// cluster of C blocks (kClusterSizes) of 16 warps, one block per SM, for its
 // whole run; one launch per cluster size and element size.
 // Device-side records of the resident engine (thin_resident.cu).
 struct ResJob {
@@ -205,10 +205,15 @@ void mosaic_release(MosaicPrepared &M, cudaStream_t stream);
 
 int cuda_status(cudaError_t e);
 
-// Resident launch groups of a batch at most: one per cluster size (1, 2, 4,
-// 8, 16) and element size (u8, u16).  Execution::enqueue needs that many helper
-// streams, and one event more.
-constexpr int kMaxResidentGroups = 10;
+// Cluster sizes of the resident engine.  3 serves images of 430 to 640 KB
+// (512^2 u16: 50 clusters of 3 fit the GPU, 36 of 4; 192 such images 23.9 ->
+// 22.5 ms).  5 and 6 were tried too: images of 0.9 to 1.3 MB are better off as
+// tiles beside larger ones (1024 uneven images 190 ms without, 200 with).
+constexpr int kClusterSizes[] = {1, 2, 3, 4, 8, 16};
+// Resident launch groups of a batch at most: one per cluster size and element
+// size (u8, u16).  Execution::enqueue needs that many helper streams, and one
+// event more.
+constexpr int kMaxResidentGroups = 2 * int(sizeof kClusterSizes / sizeof kClusterSizes[0]);
 
 // Launch groups of a batch: (cluster size, job indices) for the resident
 // engine, job indices for the tiled engine.

@@ -45,3 +45,17 @@ def test_many_cluster16_images_go_to_tiles(n):
     assert all((s["tiles_visited"] > 0) == (n >= 24) for s in stats)
     for k, t in enumerate(work):
         assert torch.equal(t, want[k % 2])
+
+
+@pytest.mark.parametrize("n", [17, 40, 60])
+@pytest.mark.parametrize("h,w,dtype", [(1030, 311, "u8"), (632, 351, "u16"), (256, 1366, "u8"), (300, 300, "u8")])
+def test_spread_clusters(h, w, dtype, n):
+    """Images that need clusters of 3 (and smaller ones), so few that each is spread over a wider cluster."""
+    img = synth.value_noise_image(h, w, dtype, seed=h + w)
+    want = torch.from_numpy(img).cuda()
+    thin.run(want, 4, kernel="tiled")
+    work = [torch.from_numpy(img).cuda() for _ in range(n)]
+    stats, rc = thin.batch(work, [4] * n)
+    assert rc == 0 and all(s["tested"] > 0 and s["converged"] == 1 for s in stats)
+    for t in work:
+        assert torch.equal(t.view(torch.uint8), want.view(torch.uint8))
