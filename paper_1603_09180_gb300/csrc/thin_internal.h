@@ -260,6 +260,12 @@ struct Execution {
 // (created once per thread and device, kept until the process exits).
 cudaError_t thread_side_streams(cudaStream_t **side, cudaEvent_t **ev);
 
+// Identity of the calling thread's current context, 0 if it cannot be had.
+unsigned long long current_context_id();
+
+// Stream-ordered device memory for a call's scratch (freed with cudaFreeAsync).
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t stream);
+
 // Raises a kernel's dynamic shared-memory cap to the device's opt-in maximum.
 // Always the same value, so host threads launching the kernel at once with
 // different shared-memory sizes never lower the cap under one another.

@@ -452,21 +452,24 @@ bool mosaic_shape(const JobSpec *jobs, int n, MosaicShape *out)
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
     const int limit = std::min(optin, per_sm / 2 - reserved) - 256;
+    // for every width the lowest tile that gives few enough tiles; of these the smallest with its halo
     double best = 0;
-    for (int tw = 32; tw <= 224; tw += 16)
-        for (int th = 16; th <= 304; th += 8) {
-            const int tiles = mosaic_tiles(jobs, n, tw, th);
-            if (tiles > 2 * sms) continue;
-            const TileLayout L = tile_layout(tw, th, halo_rows(kMaxStep), any16);
-            if (L.bytes > limit) continue;
-            const double cost = double(tw + 16) * (th + 16);
-            if (best == 0 || cost < best) {
-                best = cost;
-                out->tw = tw;
-                out->th = th;
-                out->halo = kMaxStep;
-            }
+    for (int tw = 32; tw <= 224; tw += 16) {
+        int lo = 16, hi = 304;
+        if (mosaic_tiles(jobs, n, tw, hi) > 2 * sms) continue;
+        while (lo < hi) {
+            const int mid = (lo + hi) / 16 * 8;  // a multiple of 8 below hi
+            if (mosaic_tiles(jobs, n, tw, mid) <= 2 * sms) hi = mid;
+            else lo = mid + 8;
         }
+        const double cost = double(tw + 16) * (hi + 16);
+        if ((best == 0 || cost < best) && tile_layout(tw, hi, halo_rows(kMaxStep), any16).bytes <= limit) {
+            best = cost;
+            out->tw = tw;
+            out->th = hi;
+            out->halo = kMaxStep;
+        }
+    }
     return best > 0;
 }
 
@@ -530,7 +533,7 @@ int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const t
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, L.bytes);
     if (e != cudaSuccess) return cuda_status(e);
     if (tiles > per_sm * sms) return THIN_ERR_ARG;  // the blocks wait for one another: all must be resident
-    e = async_alloc ? cudaMallocAsync(reinterpret_cast<void **>(&M->base), off, stream)
+    e = async_alloc ? scratch_alloc(reinterpret_cast<void **>(&M->base), off, stream)
                     : cudaMalloc(reinterpret_cast<void **>(&M->base), off);
     if (e != cudaSuccess) {
         cudaGetLastError();

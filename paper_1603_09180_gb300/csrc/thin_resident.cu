@@ -886,7 +886,7 @@ int resident_prepare(const JobSpec *jobs, int n, int C, const thin_options &opt,
     }
     const size_t o_x = o_ck + up(ck_words * 4);
     const size_t total = o_x + xslot * 4 * size_t(B);
-    e = async_alloc ? cudaMallocAsync(reinterpret_cast<void **>(&R->base), total, stream)
+    e = async_alloc ? scratch_alloc(reinterpret_cast<void **>(&R->base), total, stream)
                     : cudaMalloc(reinterpret_cast<void **>(&R->base), total);
     if (e != cudaSuccess) {
         cudaGetLastError();

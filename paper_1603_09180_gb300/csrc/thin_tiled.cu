@@ -590,7 +590,7 @@ int tiled_prepare(const JobSpec *jobs, int n, const thin_options &opt, cudaStrea
     const size_t total_bytes = off;
     T->total_tiles = total_tiles;
 
-    cudaError_t e = async_alloc ? cudaMallocAsync(reinterpret_cast<void **>(&T->base), total_bytes, stream)
+    cudaError_t e = async_alloc ? scratch_alloc(reinterpret_cast<void **>(&T->base), total_bytes, stream)
                                 : cudaMalloc(reinterpret_cast<void **>(&T->base), total_bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -799,37 +799,12 @@ static __device__ __align__(256) unsigned char g_thin_noalloc_scratch[THIN_NOALL
 namespace thin {
 namespace {
 
-typedef CUresult (*CtxGetCurrentFn)(CUcontext *);
-typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long *);
-
 struct NoallocSlot {
     unsigned long long ctx_id = 0;  // context the address belongs to (0: unknown)
     void *base = nullptr;
 };
 std::mutex g_noalloc_mu;
 NoallocSlot g_noalloc_slot[256];
-
-// Identity of the calling thread's current context, 0 if it cannot be had.
-unsigned long long current_context_id()
-{
-    static CtxGetCurrentFn get_current = nullptr;
-    static CtxGetIdFn get_id = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_current = reinterpret_cast<CtxGetCurrentFn>(p);
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_id = reinterpret_cast<CtxGetIdFn>(p);
-    });
-    CUcontext c = nullptr;
-    unsigned long long id = 0;
-    if (get_current && get_id && get_current(&c) == CUDA_SUCCESS && c && get_id(c, &id) == CUDA_SUCCESS) return id;
-    return 0;
-}
 
 // Device address of the scratch array on the current device (in host code the
 // array's name is only a host-side stand-in).  Looked up at the first call on
