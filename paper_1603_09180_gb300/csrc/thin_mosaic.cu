@@ -69,8 +69,9 @@ struct MosStat {
     unsigned pad;
 };
 
+// (The images travel as launch arguments: no table to copy before a run.)
 struct MosArgs {
-    const MosImage *imgs;
+    MosImage imgs[kMosaicMax];
     MosStat *st;
     unsigned *count;                // per image: kCountSlots step counters
     unsigned *flag;                 // per tile: steps published
@@ -486,8 +487,8 @@ int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const t
     const int tw = shape.tw, th = shape.th, H = shape.halo;
     const TileLayout L = tile_layout(tw, th, halo_rows(H), any16);
     std::vector<MosImage> imgs(n);
-    const size_t o_live = align_up(sizeof(MosImage) * n, 256);
-    size_t off = o_live;
+    if (n > kMosaicMax) return THIN_ERR_ARG;
+    size_t off = 0;
     const size_t o_st = off;
     off = align_up(off + sizeof(MosStat) * n, 256);
     const size_t o_err = off;
@@ -516,7 +517,7 @@ int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const t
         tiles += I.tiles_x * I.tiles_y;
     }
     off = align_up(off + sizeof(unsigned) * tiles, 256);
-    M->live_bytes = off - o_live;
+    M->live_bytes = off;
     std::vector<size_t> o_rim(2 * n), o_bits(2 * n);
     for (int k = 0; k < n; ++k)
         for (int q = 0; q < 2; ++q) {
@@ -545,8 +546,7 @@ int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const t
             imgs[k].rim[q] = reinterpret_cast<unsigned long long>(M->base + o_rim[2 * k + q]);
             imgs[k].bits[q] = reinterpret_cast<unsigned long long>(M->base + o_bits[2 * k + q]);
         }
-    e = cudaMemcpyAsync(M->base, imgs.data(), sizeof(MosImage) * n, cudaMemcpyHostToDevice, stream);  // (pageable: taken on return)
-    M->live = M->base + o_live;
+    M->live = M->base;
     M->o_st = o_st;
     M->o_err = o_err;
     M->grid = tiles;
@@ -555,7 +555,7 @@ int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const t
     M->args.resize(sizeof(MosArgs));
     MosArgs &P = *reinterpret_cast<MosArgs *>(M->args.data());
     std::memset(&P, 0, sizeof P);
-    P.imgs = reinterpret_cast<const MosImage *>(M->base);
+    std::copy(imgs.begin(), imgs.end(), P.imgs);
     P.st = reinterpret_cast<MosStat *>(M->base + o_st);
     P.error = reinterpret_cast<unsigned *>(M->base + o_err);
     P.count = reinterpret_cast<unsigned *>(M->base + o_count);
@@ -571,7 +571,7 @@ int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const t
     P.timeout_ns = 2000000000ull;
     if (const char *t = std::getenv("THIN_TIMEOUT_NS")) P.timeout_ns = std::strtoull(t, nullptr, 10);
     P.tl = L;
-    return e == cudaSuccess ? THIN_OK : cuda_status(e);
+    return THIN_OK;
 }
 
 cudaError_t mosaic_enqueue(const MosaicPrepared &M, cudaStream_t stream)
