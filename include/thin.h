@@ -88,11 +88,15 @@ typedef enum { THIN_OP_THINNING = 0, THIN_OP_SKELETON = 1 } thin_op;
  * clusters of 8 at most), or, in the wide mode, in several clusters of one
  * cooperative launch (one block per SM, clusters of 8, 4, 2 or 1 blocks,
  * whichever lets every strip be resident) that exchange boundary rows every
- * 8 phases: images up to about 30 MB.  TILED streams 64 x 32 tiles through
- * shared memory (any size).  AUTO picks RESIDENT for images that fit a
- * cluster, the wide mode for up to two larger images in a call, and TILED
- * for the rest.  NAIVE runs one launch per phase straight from global memory
- * (the reference slice). */
+ * 8 phases: images up to about 30 MB.  TILED streams tiles through shared
+ * memory (any size).  AUTO picks the mosaic engine for calls of at most 16
+ * images of one element size whose tiles all fit in shared memory at once
+ * (one image up to about 17 MB); otherwise RESIDENT for images that fit a
+ * cluster, the wide mode for up to two larger images in a call, and TILED for
+ * the rest, and for images that need clusters of 8 or 16 where a call holds
+ * many of them.  With tile_w, tile_h or halo set, AUTO uses neither the mosaic
+ * engine nor this last rule.  NAIVE runs one launch per phase straight from
+ * global memory (the reference slice). */
 typedef enum {
     THIN_KERNEL_AUTO = 0,
     THIN_KERNEL_NAIVE = 1,
@@ -103,11 +107,13 @@ typedef enum {
 typedef struct {
     int32_t rule;        /* thin_rule */
     int32_t kernel;      /* thin_kernel */
-    int32_t tile_w;      /* tiled engine: tile width in pixels, 0 = default (64); multiple of 16, 16..224 */
-    int32_t tile_h;      /* tiled engine: tile height, 0 = default (32); even, >= 8, tile_h + 2 halo <= 256 */
-    int32_t halo;        /* tiled engine: phases per tile visit = halo width, 0 = default (8); 3..8 when a u16
-                            image is in the call, else 3..16; below min(tile_w, tile_h).  A shape that does not
-                            fit one block's shared memory returns THIN_ERR_ARG */
+    int32_t tile_w;      /* tiled engine: tile width in pixels, 0 = default; multiple of 16, 16..224 */
+    int32_t tile_h;      /* tiled engine: tile height, 0 = default; even, >= 8, tile_h + 2 halo <= 256 */
+    int32_t halo;        /* tiled engine: phases per tile visit, 0 = default; 3..8 when a u16 image is in the
+                            call, else 3..16 (16 runs 15); below min(tile_w, tile_h).  A shape that does not
+                            fit one block's shared memory returns THIN_ERR_ARG.  All three 0: chosen by the
+                            images (224 x 304 or 224 x 152 and 15 phases for large ones, down to 64 x 32 and
+                            8).  One of them set: the others default to 64, 32 and 8 */
     int32_t reserved;    /* 0.  Test hook: 1 makes block 0 of the tiled engine skip its first grid barrier, so
                             that the bounded wait runs out and the call reports THIN_ERR_TIMEOUT */
     int64_t start_phase; /* global phase index of the first phase (resume), >= 0 */
@@ -162,12 +168,15 @@ typedef struct {
 
 /*
  * Lambda-thin n independent images of any sizes, dtypes and lambdas in one
- * call.  Images that fit one thread-block cluster's shared memory run on the
- * resident engine, one launch per cluster size, the launches side by side
- * on streams forked from `stream` and joined back into it.  Images too large
- * for a cluster run in the wide resident mode, one launch each, when there
- * are at most two of them (any number with THIN_KERNEL_RESIDENT); otherwise
- * they go to one persistent launch of the tiled engine, after the resident
+ * call.  A call of at most 16 images of one element size goes to one launch
+ * of the mosaic engine where their tiles fit.  Otherwise images that fit one
+ * thread-block cluster's shared memory run on the resident engine, one launch
+ * per cluster size, the launches side by side on streams forked from `stream`
+ * and joined back into it.  Images too large for a cluster run in the wide
+ * resident mode, one launch each, when there are at most two of them (any
+ * number with THIN_KERNEL_RESIDENT); otherwise they, and many images that need
+ * clusters of 8 or 16 (24 of 16 blocks, 64 of 8, or 32 beside the former), go
+ * to one persistent launch of the tiled engine, after the resident
  * launches.  Every such launch loops on the device until its images are
  * stable.  THIN_KERNEL_TILED sends every image to the tiled engine;
  * THIN_KERNEL_NAIVE thins the images one after another, as thin_run does
@@ -186,10 +195,10 @@ int thin_batch(const thin_job *jobs, int n, thin_adj adj, void *stream, const th
  * thin_plan_create does all host work of a thin_batch call once (checks,
  * launch groups, device job tables, tensor maps) and captures the device
  * work of one run into a CUDA graph: per-run resets, the resident engine's
- * launch groups side by side, the tiled engine after them.  Images that go
- * to the tiled engine get a tile shape and halo depth chosen by
- * thin_autotune on the largest of them, unless opt sets tile_w, tile_h or
- * halo.
+ * launch groups side by side, the mosaic or tiled engine after them.  Images
+ * that go to the tiled engine get its large tiles where these fill the GPU,
+ * else a tile shape and halo depth chosen by thin_autotune on the largest of
+ * them, unless opt sets tile_w, tile_h or halo.
  * thin_plan_launch enqueues that graph: every image is thinned in place, with
  * exactly the result thin_batch gives.  The images must stay at the same
  * device addresses while the plan exists; relaunching thins whatever the
@@ -228,8 +237,8 @@ int thin_plan_destroy(thin_plan *p);
  * (8,4) adjacency, whichever pair the image is later thinned with.
  * trial_phases bounds each trial (< 0: every trial runs to stability).
  * best_ms (may be NULL) receives the winner's time.  Synchronous.
- * Candidates: 64x32 (h 8, 6, 4), 128x32, 64x64, 128x64, 32x32, 96x48,
- * 128x16, 224x32, 48x64 (h 8), 64x16 (h 6).  THIN_ERR_ARG for an image
+ * Candidates: 224x240, 224x160, 224x96, 160x96, 128x128, 128x64, 96x96,
+ * 96x48, 64x64, 64x32 (h 8), 128x64, 64x32 (h 6).  THIN_ERR_ARG for an image
  * without interior points.
  */
 int thin_autotune(const void *img_dev, int w, int h, size_t pitch_bytes, thin_dtype dt, uint32_t lambda,
@@ -269,8 +278,8 @@ void thin_point_table_adj(thin_adj adj, uint32_t out[256]);
  * device memory; every GPU that loads the library holds it until the process
  * exits.  The call allocates nothing.
  *   - An image whose scratch (a second image-sized buffer, one more if its
- *     rows are not 16-byte aligned, 4 bytes per 8 x 2 pixels of change stamps
- *     and a few words per 64 x 32 tile) does not fit returns
+ *     rows are not 16-byte aligned, 2 bytes per 8 x 2 pixels of dirty bits
+ *     and a few words per tile) does not fit returns
  *     THIN_ERR_TOO_LARGE and is left untouched.  16 MiB holds, for example,
  *     a 3500 x 3500 u8 or a 2500 x 2500 u16 image with 16-byte aligned rows
  *     (unaligned rows need the extra buffer: 2048 x 2048 u8 still fits).
@@ -305,7 +314,8 @@ const char *thin_version(void);
  * time take from the large queue, and each of their tiled launches uses at
  * most a quarter of the SMs, so small requests keep running beside them.
  * The lane allocates the device images, copies them in and launches them as
- * one batch (never the wide mode, so that the lanes share the GPU).  Each
+ * one batch (never the wide mode or the mosaic engine, so that the lanes
+ * share the GPU).  Each
  * resident image is retired as soon as it is finished -- its result copied
  * back and its bytes and slot returned -- while the rest of its batch still
  * runs; tiled images retire when their batch ends.  Queued requests are

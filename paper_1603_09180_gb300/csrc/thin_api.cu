@@ -156,7 +156,10 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     G->wide.clear();
     G->mosaic.clear();
     G->tiled.clear();
-    if (allow_wide && o.kernel == THIN_KERNEL_AUTO && n <= kMosaicMax && mosaic_shape(specs.data(), n, &G->mosaic_tile)) {
+    // (a call that sets a tile shape has it checked where images go to the tiled engine: it keeps that route)
+    const bool own_tiles = o.tile_w || o.tile_h || o.halo;
+    if (allow_wide && o.kernel == THIN_KERNEL_AUTO && !own_tiles && n <= kMosaicMax &&
+        mosaic_shape(specs.data(), n, &G->mosaic_tile)) {
         for (int k = 0; k < n; ++k) G->mosaic.push_back(k);
         return THIN_OK;
     }
@@ -177,7 +180,7 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     // resident 262 / 221 / 202 ms.  (Serving, which passes allow_wide = false,
     // keeps them resident: its small lanes retire image by image.  So does a call
     // that sets a tile shape, which not every image may take.)
-    if (allow_wide && o.kernel == THIN_KERNEL_AUTO && !o.tile_w && !o.tile_h && !o.halo) {
+    if (allow_wide && o.kernel == THIN_KERNEL_AUTO && !own_tiles) {
         int count[17] = {};
         for (int k = 0; k < n; ++k) ++count[cls[k]];
         const int huge = count[0] > kWideMax ? count[0] : 0;

@@ -49,3 +49,12 @@ def test_few_images(n):
         ref, rst = oracle.thin(a, lam)
         assert np.array_equal(t.cpu().numpy(), ref)
         assert st["lowered"] == rst["lowered"] and st["last_change_phase"] == rst["last_change_phase"]
+
+
+def test_set_tile_shape_is_still_checked():
+    """Images that fit the mosaic's tiles but no cluster, with a depth that no u16 call takes: refused, untouched."""
+    img = synth.value_noise_image(1500, 1500, "u16", seed=1)
+    work = [torch.from_numpy(img).cuda() for _ in range(3)]
+    with pytest.raises(thin.ThinError):
+        thin.batch(work, [60] * 3, halo=9)
+    assert all(np.array_equal(t.cpu().numpy(), img) for t in work)
