@@ -187,10 +187,11 @@ void tiled_defaults(int dtype, int *tw, int *th, int *halo);
 // memory at once, one block to a tile.
 // A call of at most this many images (of one element size) goes to the mosaic
 // engine where their tiles fit: it spreads an image over far more SMs than a
-// cluster has, with no barrier over the grid.  Resident against mosaic, one
-// image: 512^2 u8 at lambda = 20 3.9 / 2.3 ms, 1000^2 13.1 / 4.6, 2048^2 at
-// lambda = 30 (wide) 21.6 / 10.2, 4096^2 35.1 / 32.0, 64^2 0.28 / 0.26; 16 images
-// of 512^2 6.7 / 5.5, of 200^2 1.82 / 1.59; 32 images 7.1 / 7.2 and 1.81 / 1.88.
+// cluster has, with no barrier over the grid.  Resident against mosaic (tiles in
+// all block slots), one image: 512^2 u8 at lambda = 20 3.9 / 2.3 ms, 1000^2
+// 13.1 / 4.6, 2048^2 at lambda = 30 (wide) 21.6 / 10.2, 4096^2 35.1 / 32.0, 64^2
+// 0.28 / 0.26; 16 images of 512^2 6.7 / 5.5, of 200^2 1.82 / 1.59; 32 images
+// 7.1 / 7.2 and 1.81 / 1.88.
 constexpr int kMosaicMax = 16;
 struct MosaicShape {
     int tw, th, halo;  // tile, phases per step

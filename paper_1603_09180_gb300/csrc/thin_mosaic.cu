@@ -35,6 +35,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <type_traits>
@@ -441,6 +442,18 @@ int mosaic_tiles(const JobSpec *jobs, int n, int tw, int th)
 
 }  // namespace
 
+// How many tiles: about one for every 10 pixels of an image's side (the root of
+// its area), so that a whole number of such calls fill the block slots.  Small
+// tiles gain little, since each also tests its ring, and calls on other streams
+// run beside this one only if their blocks all fit.  One call, and 16 calls on
+// 16 streams, in ms, on the clusters and the wide mode / with tiles in all slots /
+// by this rule (u8): 512^2 at lambda = 0 0.56 / 0.22 / 0.22 and 1.54 / 2.95 /
+// 0.91, at lambda = 20 6.9 / 2.7 / 2.9 and 10.6 / 39.2 / 8.9; 256^2 3.1 / 1.4 /
+// 1.55 and 5.9 / 11.4 / 3.6; 1000^2 17.4 / 5.0 / 5.3 and 33.9 / 79.6 / 33.3;
+// 2048^2 at lambda = 30 30.0 / 11.7 / 13.2 and 173 / 188 / 122; 4 batches of 4
+// 512^2 images on 4 streams 10.3 / 13.8 / 7.8.  A tile every 8 or 12 pixels: one
+// call 4 % less or 6 % more, 16 at once 30 % more or 8 % less.  (Long strips need
+// more tiles than that: all slots.)
 bool mosaic_shape(const JobSpec *jobs, int n, MosaicShape *out)
 {
     const bool any16 = jobs[0].dtype == THIN_U16;
@@ -453,25 +466,31 @@ bool mosaic_shape(const JobSpec *jobs, int n, MosaicShape *out)
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
     const int limit = std::min(optin, per_sm / 2 - reserved) - 256;
-    // for every width the lowest tile that gives few enough tiles; of these the smallest with its halo
-    double best = 0;
-    for (int tw = 32; tw <= 224; tw += 16) {
-        int lo = 16, hi = 304;
-        if (mosaic_tiles(jobs, n, tw, hi) > 2 * sms) continue;
-        while (lo < hi) {
-            const int mid = (lo + hi) / 16 * 8;  // a multiple of 8 below hi
-            if (mosaic_tiles(jobs, n, tw, mid) <= 2 * sms) hi = mid;
-            else lo = mid + 8;
+    const int slots = 2 * sms;
+    double want = 0;
+    for (int k = 0; k < n; ++k) want += std::max(std::sqrt(double(jobs[k].w) * jobs[k].h) / 10, 8.0);
+    for (int most : {slots / std::max(int(slots / want + 0.6), 1), slots}) {
+        // for every width the lowest tile that gives few enough tiles; of these the smallest with its halo
+        double best = 0;
+        for (int tw = 32; tw <= 224; tw += 16) {
+            int lo = 16, hi = 304;
+            if (mosaic_tiles(jobs, n, tw, hi) > most) continue;
+            while (lo < hi) {
+                const int mid = (lo + hi) / 16 * 8;  // a multiple of 8 below hi
+                if (mosaic_tiles(jobs, n, tw, mid) <= most) hi = mid;
+                else lo = mid + 8;
+            }
+            const double cost = double(tw + 16) * (hi + 16);
+            if ((best == 0 || cost < best) && tile_layout(tw, hi, halo_rows(kMaxStep), any16).bytes <= limit) {
+                best = cost;
+                out->tw = tw;
+                out->th = hi;
+                out->halo = kMaxStep;
+            }
         }
-        const double cost = double(tw + 16) * (hi + 16);
-        if ((best == 0 || cost < best) && tile_layout(tw, hi, halo_rows(kMaxStep), any16).bytes <= limit) {
-            best = cost;
-            out->tw = tw;
-            out->th = hi;
-            out->halo = kMaxStep;
-        }
+        if (best > 0) return true;
     }
-    return best > 0;
+    return false;
 }
 
 int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const thin_options &opt, cudaStream_t stream,

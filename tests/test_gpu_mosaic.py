@@ -17,7 +17,7 @@ pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(),
 @pytest.mark.parametrize("h,w,dtype,lam,op,adj", [
     (3, 3, "u8", 4, "thinning", 0), (16, 32, "u8", 0, "thinning", 0), (17, 33, "u16", 60, "thinning", 0),
     (128, 256, "u8", 12, "thinning", 0), (129, 257, "u8", 12, "skeleton", 0), (33, 700, "u16", 200, "thinning", 1),
-    (600, 35, "u8", 0, "skeleton", 1)])
+    (600, 35, "u8", 0, "skeleton", 1), (3, 30000, "u8", 8, "thinning", 0), (511, 513, "u8", 3, "thinning", 0)])
 def test_mosaic(h, w, dtype, lam, op, adj):
     img = synth.value_noise_image(h, w, dtype, seed=2 * h + w)
     ref, rst = oracle.thin(img, lam, op={"thinning": 0, "skeleton": 1}[op], adj=adj)
