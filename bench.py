@@ -16,8 +16,8 @@ latency, and the single-image service time of the mix).
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
   python bench.py --workload large|uneven|serve   (the other configurations)
 
---workload large: the large images with the tiled engine beside the wide
-resident mode and a halo sweep.  --workload uneven: 1024 u8 images with
+--workload large: the large images with the tiled engine beside the default
+engine and a halo sweep.  --workload uneven: 1024 u8 images with
 sides log-uniform in [64, 2048] and lambda in {0, 10, 25}, one thin_batch
 call against one thin_run call per image.  --workload serve: Poisson
 arrivals of u8/u16 images with sides log-uniform in [128, 4096] through the
@@ -57,7 +57,7 @@ TRAFFIC_FILE = os.path.join(ROOT, "profiles", "roofline_traffic.json")
 
 # The sources of the dominant kernel (k_resident): its recorded DRAM traffic is used only while
 # these are unchanged since the ncu capture.
-KERNEL_SOURCES = ("thin_resident.cu", "thin_simd.cuh", "thin_common.cuh", "thin_internal.h")
+KERNEL_SOURCES = ("thin_resident.cu", "thin_block.cuh", "thin_simd.cuh", "thin_common.cuh", "thin_internal.h")
 
 
 def kernel_source_hash() -> str:
@@ -550,7 +550,7 @@ def large_specs():
 
 def large_measure(imgs, steps, warmup, flush, stream, compare_tiled=False, halo_sweep=False):
     """4096^2 u8 and 8192^2 u16 at lambda 0 and 30 on the default engine (thin_run): ms, sweep rates over
-    active and over all pixels, and the HBM roofline (2 sizeof(T) bytes per active pixel-round)."""
+    tested and over all pixels, and the HBM roofline (2 sizeof(T) bytes per active pixel-round)."""
     import torch
     from paper_1603_09180_gb300 import thin
     dev = flush.device
@@ -562,15 +562,13 @@ def large_measure(imgs, steps, warmup, flush, stream, compare_tiled=False, halo_
         es = work.element_size()
         for lam in lams:
             work.copy_(pristine)
-            st = thin.run(work, lam)  # the default engine: wide resident if the image fits, else tiled
-            engine = "tiled" if st["tiles_visited"] else "resident (wide)"
-            tw, th, H = 64, 32, 8
+            st = thin.run(work, lam)  # the default engine: mosaic if the image's tiles fit, else tiled
+            engine = "tiled" if st["tiles_visited"] else "mosaic"
             ms = _timed(lambda: thin.run(work, lam, stats=False), lambda: work.copy_(pristine),
                         flush, stream, steps, warmup)
             t = statistics.median(ms) / 1e3
-            # pixel-rounds over active tiles (tiled) or tested pixel-rounds (resident: a point is tested
-            # at most once per round, and only while a neighbour moved)
-            active = st["tiles_visited"] * tw * th * H / 4.0 if st["tiles_visited"] else float(st["tested"])
+            # tested pixel-rounds: a point is tested at most once per round, and only while a neighbour moved
+            active = float(st["tested"])
             full = w * h * st["phases"] / 4.0
             r = {"image": "%dx%d %s" % (w, h, dt), "lambda": lam, "engine": engine, "ms": round(t * 1e3, 3),
                  "phases": st["phases"], "tiles_visited": st["tiles_visited"], "tested": st["tested"],
@@ -599,7 +597,7 @@ def large_measure(imgs, steps, warmup, flush, stream, compare_tiled=False, halo_
 
 
 def run_large(args):
-    """Large single images on the default engine (the wide resident mode or the tiled engine)."""
+    """Large single images on the default engine (the mosaic or the tiled engine)."""
     import torch
     from paper_1603_09180_gb300 import thin
     imgs = _gen_pool(large_specs(), 2)
@@ -616,12 +614,10 @@ def run_large(args):
             "unit": "Gpix-sweeps/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
             "higher_is_better": True, "dtype": "u8/u16", "data": "synthetic", "workload": "large",
             "config": {"workload": "4096x4096 u8 and 8192x8192 u16 (0..4095), lambda 0 and 30, default engine "
-                                   "(wide resident where the image fits the GPU's shared memory, else tiled 64x32, "
-                                   "halo 8)", "l2": "flushed before every timed run"},
+                                   "(mosaic where the image's tiles fit the GPU's shared memory, else tiled)", "l2": "flushed before every timed run"},
             "roofline": {"bound": "hbm", "achieved": head["achieved_gbs"], "peak": peak, "unit": "GB/s",
                          "frac": head["frac"], "peak_source": src,
-                         "note": "2 B (u8) or 4 B (u16) per pixel-round over active tiles (tiled) or per tested "
-                                 "pixel-round (resident)"},
+                         "note": "2 B (u8) or 4 B (u16) per tested pixel-round"},
             "cases": results, "clocks": clk.summary()}
 
 
