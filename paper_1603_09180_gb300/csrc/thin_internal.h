@@ -167,8 +167,8 @@ int resident_wide_strips(int w, int h, int dtype, size_t smem_limit, int *c_out)
 
 // A tiled launch prepared on the host (opaque; thin_tiled.cu).
 struct TiledPrepared;
-// max_grid > 0 caps the launch at that many blocks (serving keeps the rest of
-// the GPU free for the resident launches of its other lanes).
+// max_grid > 0 caps the launch at that many blocks of 8 warps (serving keeps the
+// rest of the GPU free for the resident launches of its other lanes).
 int tiled_prepare(const JobSpec *jobs, int n, const thin_options &opt, cudaStream_t stream, bool async_alloc,
                   TiledPrepared **out, int max_grid = 0);
 cudaError_t tiled_enqueue(const TiledPrepared *T, cudaStream_t stream);

@@ -393,7 +393,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_mosaic(MosArgs P)
             __syncthreads();
         }
         int chg_j = -1;
-        visit_phases<typename std::conditional<ES == 1, uint8_t, uint16_t>::type>(L, smem, V, rule, nlow, ntest, chg_j);
+        visit_phases<typename std::conditional<ES == 1, uint8_t, uint16_t>::type, kThreads>(L, smem, V, rule, nlow, ntest,
+                                                                                          chg_j);
         if (chg_j >= 0) last = g0 + chg_j;
         g0 += V.Hs;
         ++s;

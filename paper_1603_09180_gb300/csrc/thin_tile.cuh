@@ -98,8 +98,9 @@ static_assert(sizeof(TileCtrl) <= kOffBar - kOffCtrl, "control words overlap the
 // Hs phases of the subfield schedule on a staged tile.  Staged column 0 is
 // image column x0 - kPadCols, staged row 0 image row y0 - hr.  Phase j updates
 // the points of its parity within distance Hs - j of the tile and off the image
-// border; after Hs phases the tile and its dirty bits are exact.
-template <typename T>
+// border; after Hs phases the tile and its dirty bits are exact.  A bitmap has at
+// most a word per thread.
+template <typename T, int THREADS>
 __device__ __forceinline__ void visit_phases(const TileLayout &L, uint8_t *smem, const Visit &V, const PointRule &rule,
                                              int &nlow, int &ntest, int &chg_j)
 {
@@ -119,7 +120,7 @@ __device__ __forceinline__ void visit_phases(const TileLayout &L, uint8_t *smem,
     map.own_col = kPadCols / 8;
     map.own_cols = V.tw / 8;
     // this thread's piece of a bitmap: a byte, or 16 or 32 bits where there are more of them than threads
-    const int unit = words * 4 <= kThreads ? 0 : words * 2 <= kThreads ? 1 : 2;
+    const int unit = words * 4 <= THREADS ? 0 : words * 2 <= THREADS ? 1 : 2;
     const int pword = int(threadIdx.x) >> (2 - unit), pshift = (int(threadIdx.x) << (3 + unit)) & 31;
     const uint32_t pones = unit == 0 ? 0xffu : unit == 1 ? 0xffffu : 0xffffffffu;
     for (int j = 0; j < V.Hs; ++j) {
@@ -152,7 +153,7 @@ __device__ __forceinline__ void visit_phases(const TileLayout &L, uint8_t *smem,
         __syncthreads();
         const int N = int(*reinterpret_cast<volatile unsigned *>(&ctrl->qn[j & 1]));
         if (threadIdx.x == 0) ctrl->qn[(j + 1) & 1] = 0u;  // last read in the previous phase
-        if (work_queue<T, kThreads>(map, rule, queue, N, px, py, xlo, xhi, nlow, ntest)) chg_j = j;
+        if (work_queue<T, THREADS>(map, rule, queue, N, px, py, xlo, xhi, nlow, ntest)) chg_j = j;
         __syncthreads();
     }
 }

@@ -196,6 +196,7 @@ __device__ __forceinline__ int find_image(const ImgDesc *imgs, int n, int gt)
 }
 
 // Stores the tile (clipped to the image) to `dst`, a row of which is 16-byte aligned.
+template <int THREADS>
 __device__ __forceinline__ void tile_store(const uint8_t *tile, int row_bytes, int es, const Visit &V, char *dst, size_t pitch)
 {
     const int cw = min(V.tw, V.w - V.x0) * es, ch = min(V.th, V.h - V.y0);
@@ -203,7 +204,7 @@ __device__ __forceinline__ void tile_store(const uint8_t *tile, int row_bytes, i
     const uint32_t M = div_magic(vpr);
     char *base = dst + size_t(V.y0) * pitch + size_t(V.x0) * es;
     const uint8_t *src = tile + V.hr * row_bytes + kPadCols * es;
-    for (int v = threadIdx.x; v < ch * vpr; v += kThreads) {
+    for (int v = threadIdx.x; v < ch * vpr; v += THREADS) {
         const int row = div_small(v, vpr, M), col = (v - row * vpr) * 16;
         char *d = base + size_t(row) * pitch + col;
         const uint8_t *s = src + row * row_bytes + col;
@@ -224,8 +225,10 @@ __device__ __forceinline__ void decode(const EngineArgs &P, bool full, const uns
     tx = local - ty * D.tiles_x;
 }
 
-__global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 2 * kWarps / WARPS) k_engine(EngineArgs P)
 {
+    constexpr int THREADS = 32 * WARPS;
     extern __shared__ __align__(128) uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
     __shared__ int s_flag;
@@ -298,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
                 const int gx = (V.x0 - kPadCols) / 8 + lane, gy0 = (V.y0 - HR) / 2;  // (both exact: multiples of 8 and 2)
                 const bool col = lane < (P.tw + 2 * kPadCols) / 8 && gx >= 0 && gx < D.cells_x;
 #pragma unroll 4
-                for (int cr = warp; cr < words; cr += kWarps) {
+                for (int cr = warp; cr < words; cr += WARPS) {
                     const int gy = gy0 + cr;
                     unsigned v = 0;
                     if (col && gy >= 0 && gy < D.cells_y) v = __ldcg(bits + size_t(gy) * D.cells_x + gx);
@@ -318,9 +321,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
             const PointRule rule = point_rule(smem, P.rule | (D.adj << 2), D.lam, es, true);  // F^- reading, operator, pair
             TileLayout Li = L;
             Li.row_bytes = (P.tw + 2 * kPadCols) * es;
-            if (u16) visit_phases<uint16_t>(Li, smem, V, rule, nlow, ntest, chg_j);
-            else visit_phases<uint8_t>(Li, smem, V, rule, nlow, ntest, chg_j);
-            tile_store(tile, Li.row_bytes, es, V, reinterpret_cast<char *>(D.buf[src ^ 1]), D.pitch);
+            if (u16) visit_phases<uint16_t, THREADS>(Li, smem, V, rule, nlow, ntest, chg_j);
+            else visit_phases<uint8_t, THREADS>(Li, smem, V, rule, nlow, ntest, chg_j);
+            tile_store<THREADS>(tile, Li.row_bytes, es, V, reinterpret_cast<char *>(D.buf[src ^ 1]), D.pitch);
             // the tile's dirty bits, and which neighbours they can reach in the next step
             {
                 unsigned char *bits = reinterpret_cast<unsigned char *>(D.cells[src ^ 1]);
@@ -329,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_engine(EngineArgs P)
                 const int zx = (H + 2 + 7) / 8, zy = (H + 2 + 1) / 2;  // cells within reach of an edge
                 const unsigned left = 0xffffffffu >> (32 - min(zx, 32)), right = left << max(cols - zx, 0);
                 unsigned near = 0;
-                for (int cr = warp; cr < rows; cr += kWarps) {
+                for (int cr = warp; cr < rows; cr += WARPS) {
                     const int gy = gy0 + cr;
                     const uint32_t *w = dirty + HR / 2 + cr;
                     const int b = lane + kPadCols / 8;
@@ -433,6 +436,38 @@ EncodeTiledFn encode_fn()
     return fn;
 }
 
+// The kernel's builds.  Blocks of fewer warps leave room for more of them on an
+// SM (16 warps in all): small tiles, which only a caller or the autotuner sets,
+// give a phase too few groups for 8 warps.
+struct EngineBuild {
+    const void *kernel;
+    int warps;
+};
+const EngineBuild kBuilds[3] = {{reinterpret_cast<const void *>(k_engine<8>), 8},
+                                {reinterpret_cast<const void *>(k_engine<4>), 4},
+                                {reinterpret_cast<const void *>(k_engine<2>), 2}};
+
+// The build for a launch: with n warps a block where 16 / n blocks fit an SM's
+// shared memory and there are tiles enough, one for each of those blocks (4
+// warps) or four (2 warps).  4096^2 u8 at lambda = 10 with 8 / 4 / 2 warps: tiles
+// of 32 x 32 and 8 phases 165 / 110 / 94 ms, 64 x 32 110 / 79 / 74, 64 x 64 83 /
+// 68 / 73, 128 x 64 64 / 57 / 74 (with a warp to a tile of 64 x 32, all points
+// tested, 97).  1000^2, 64 x 32 (512 tiles): 9.5 / 9.4 / 11.8 ms, 32 x 32 (1024)
+// 11.1 / 10.5 / 12.4.
+const EngineBuild &engine_build(int tiles, const TileLayout &L, int smem, int sms)
+{
+    int dev = 0, per_sm = 0, reserved = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    const auto fits = [&](int warps) {
+        return L.rows / 2 <= 32 * warps && smem + 256 + reserved <= per_sm * warps / (2 * kWarps);
+    };
+    if (tiles >= 32 * sms && fits(2)) return kBuilds[2];
+    if (tiles >= 4 * sms && fits(4)) return kBuilds[1];
+    return kBuilds[0];
+}
+
 // Tile shape and phases per step.  What the caller set is taken as it is (and
 // checked); with nothing set the largest of these shapes that still gives every
 // SM two tiles: a large tile has less halo (224 x 152 with rings of 1 to 15:
@@ -496,6 +531,7 @@ void tiled_defaults(int dtype, int *tw, int *th, int *halo)
 // stats/control words uploaded into one device allocation.
 struct TiledPrepared {
     int n = 0, H = 0, grid = 0, smem = 0;
+    EngineBuild build = {nullptr, 0};
     bool async_alloc = true;
     char *base = nullptr;
     size_t o_stat = 0, o_ctl = 0, o_stat0 = 0, o_ctl0 = 0, o_listed = 0, o_cells = 0, cells_bytes = 0;
@@ -659,23 +695,25 @@ int tiled_prepare(const JobSpec *jobs, int n, const thin_options &opt, cudaStrea
     P.debug = opt.reserved;
     P.tl = TL;
     T->smem = 128 + TL.bytes;
+    T->build = engine_build(total_tiles, TL, T->smem, sms);
     {
         int optin = 0;
         cudaFuncAttributes fa;
         if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-            cudaFuncGetAttributes(&fa, reinterpret_cast<const void *>(k_engine)) == cudaSuccess &&
+            cudaFuncGetAttributes(&fa, T->build.kernel) == cudaSuccess &&
             size_t(T->smem) + fa.sharedSizeBytes > size_t(optin)) {
             tiled_release(T, stream);
             return THIN_ERR_ARG;  // this tile shape and halo do not fit one block's shared memory
         }
     }
 
-    if (e == cudaSuccess) e = allow_max_dynamic_smem(reinterpret_cast<const void *>(k_engine));
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(T->build.kernel);
     int per_sm = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_engine, kThreads, T->smem);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, T->build.kernel, 32 * T->build.warps, T->smem);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
     T->grid = std::max(1, std::min(sms * per_sm, total_tiles));
-    if (max_grid > 0) T->grid = std::min(T->grid, max_grid);
+    if (max_grid > 0) T->grid = std::min(T->grid, max_grid * kWarps / T->build.warps);
     if (opt.reserved == 1) T->grid = std::max(T->grid, std::min(2, sms * per_sm));
     if (e != cudaSuccess) {
         tiled_release(T, stream);
@@ -705,8 +743,7 @@ cudaError_t tiled_enqueue(const TiledPrepared *T, cudaStream_t stream)
     if (e == cudaSuccess) e = cudaMemsetAsync(base + T->o_cells, 0x0f, T->cells_bytes, stream);  // every group dirty
     if (e == cudaSuccess) {
         void *args[] = {const_cast<EngineArgs *>(&T->P)};
-        e = cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_engine), dim3(T->grid), dim3(kThreads), args, T->smem,
-                                        stream);
+        e = cudaLaunchCooperativeKernel(T->build.kernel, dim3(T->grid), dim3(32 * T->build.warps), args, T->smem, stream);
     }
     if (e == cudaSuccess) {
         k_copy_out<<<dim3(64, T->n), 256, 0, stream>>>(T->P.imgs, T->P.st, T->n);
@@ -963,16 +1000,19 @@ int tiled_run_noalloc(const JobSpec &J, const thin_options &opt, cudaStream_t st
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, reinterpret_cast<const void *>(k_engine));
+    const EngineBuild build = engine_build(total_tiles, TL, smem, sms);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, build.kernel);
     if (e == cudaSuccess && size_t(smem) + fa.sharedSizeBytes > size_t(optin)) return THIN_ERR_ARG;
-    if (e == cudaSuccess) e = allow_max_dynamic_smem(reinterpret_cast<const void *>(k_engine));
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_engine, kThreads, smem);
+    // (every build, so that the first call loads them all and a later one of another size maps nothing)
+    for (const EngineBuild &b : kBuilds)
+        if (e == cudaSuccess) e = allow_max_dynamic_smem(b.kernel);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build.kernel, 32 * build.warps, smem);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
     const int grid = std::max(1, std::min(sms * per_sm, total_tiles));
     if (e == cudaSuccess) {
         void *args[] = {&P};
-        e = cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_engine), dim3(grid), dim3(kThreads), args, smem,
-                                        stream);
+        e = cudaLaunchCooperativeKernel(build.kernel, dim3(grid), dim3(32 * build.warps), args, smem, stream);
     }
     if (e == cudaSuccess) {
         k_copy_out<<<dim3(64, 1), 256, 0, stream>>>(P.imgs, P.st, 1);

@@ -30,6 +30,21 @@ def test_tiles(h, w, dtype, lam, tile, halo):
     assert np.array_equal(t.cpu().numpy(), ref)
 
 
+@pytest.mark.parametrize("op,adj", [("thinning", 0), ("skeleton", 1)])
+@pytest.mark.parametrize("h,w,dtype,tile,halo", [
+    (759, 1009, "u8", (32, 32), 8), (1601, 805, "u16", (64, 32), 4), (789, 785, "u8", (16, 8), 3), (785, 789, "u16", (16, 8), 3),
+    (1800, 1501, "u8", (32, 16), 15), (1220, 515, "u8", (32, 32), 16)])
+def test_many_small_tiles(h, w, dtype, tile, halo, op, adj):
+    """So many tiles that blocks of 4 or of 2 warps take them."""
+    img = synth.value_noise_image(h, w, dtype, seed=h)
+    lam = 0 if dtype == "u8" else 40
+    ref, rst = oracle.thin(img, lam, op={"thinning": 0, "skeleton": 1}[op], adj=adj)
+    t = torch.from_numpy(img).cuda()
+    st = thin.run(t, lam, kernel="tiled", tile=tile, halo=halo, op=op, adj=adj)
+    assert np.array_equal(t.cpu().numpy(), ref)
+    assert st["converged"] == 1 and st["lowered"] == rst["lowered"] and st["last_change_phase"] == rst["last_change_phase"]
+
+
 @pytest.mark.parametrize("n", [23, 24])
 def test_many_cluster16_images_go_to_tiles(n):
     """24 images that need a cluster of 16 blocks go to the tiled engine, 23 do not; the result is the same."""
