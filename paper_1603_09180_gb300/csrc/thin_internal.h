@@ -9,6 +9,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/thin.h"
+#include "thin_layout.h"
 
 namespace thin {
 
@@ -193,9 +194,6 @@ void tiled_defaults(int dtype, int *tw, int *th, int *halo);
 // 0.28 / 0.26; 16 images of 512^2 6.7 / 5.5, of 200^2 1.82 / 1.59; 32 images
 // 7.1 / 7.2 and 1.81 / 1.88.
 constexpr int kMosaicMax = 16;
-struct MosaicShape {
-    int tw, th, halo;  // tile, phases per step
-};
 // The best tile shape for these images; false if they do not fit.
 bool mosaic_shape(const JobSpec *jobs, int n, MosaicShape *out);
 struct MosaicPrepared {

@@ -192,19 +192,20 @@ __device__ __noinline__ void fetch_rims(uint8_t *smem, unsigned step)
     const bool in_row = v < inner + es && (left || v >= 0) && (right || v < inner);
     const char *from = rim + (t.x0 * es + 16 * v);
     uint8_t *to = tile + kPadCols * es + 16 * v;
-    uint4 row[4], side[3];
+    constexpr int kSide = mosaic_side_turns(ES);
+    uint4 row[4], side[kSide];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const int r = warp + q * kWarps, y = r < HR ? r - HR : t.th + r - HR;
         if (r < 2 * HR && in_row && (r < HR ? above : below))
             row[q] = __ldcg(reinterpret_cast<const uint4 *>(from + (long long)(t.y0 + y) * t.rim_pitch));
     }
-    // columns left and right: es vectors a side and row (2 es t.th <= 608)
+    // columns left and right: es vectors a side and row, of every row
     const int side_shift = es, side_q = tid & (2 * es - 1);
     const bool side_have = side_q >= es ? right : left;
     const int side_x = side_q >= es ? 16 * (inner + side_q - es) : 16 * (side_q - es);
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
+    for (int q = 0; q < kSide; ++q) {
         const int y = (tid + q * kThreads) >> side_shift;
         if (y < t.th && side_have)
             side[q] = __ldcg(reinterpret_cast<const uint4 *>(rim + (size_t(t.y0 + y) * t.rim_pitch + t.x0 * es + side_x)));
@@ -215,7 +216,7 @@ __device__ __noinline__ void fetch_rims(uint8_t *smem, unsigned step)
         if (r < 2 * HR && in_row && (r < HR ? above : below)) *reinterpret_cast<uint4 *>(to + (y + HR) * t.row_bytes) = row[q];
     }
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
+    for (int q = 0; q < kSide; ++q) {
         const int y = (tid + q * kThreads) >> side_shift;
         if (y < t.th && side_have)
             *reinterpret_cast<uint4 *>(tile + (y + HR) * t.row_bytes + kPadCols * es + side_x) = side[q];
@@ -266,7 +267,7 @@ __device__ __noinline__ uint32_t publish_rim(uint8_t *smem, unsigned step)
     }
     const int q0 = tid & (2 * es - 1), x0 = q0 >= es ? 16 * (inner - 2 * es + q0) : 16 * q0;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
+    for (int q = 0; q < mosaic_side_turns(ES); ++q) {
         const int y = (tid + q * kThreads) >> es;
         if (y >= HR && y < t.th - HR)
             __stcg(reinterpret_cast<uint4 *>(dst + size_t(y) * t.rim_pitch + x0),
@@ -434,27 +435,8 @@ const void *mosaic_kernel(int es)
     return es == 2 ? reinterpret_cast<const void *>(k_mosaic<2>) : reinterpret_cast<const void *>(k_mosaic<1>);
 }
 
-int mosaic_tiles(const JobSpec *jobs, int n, int tw, int th)
-{
-    long long t = 0;
-    for (int k = 0; k < n; ++k) t += (long long)((jobs[k].w + tw - 1) / tw) * ((jobs[k].h + th - 1) / th);
-    return int(std::min<long long>(t, 1 << 30));
-}
-
 }  // namespace
 
-// How many tiles: about one for every 10 pixels of an image's side (the root of
-// its area), so that a whole number of such calls fill the block slots.  Small
-// tiles gain little, since each also tests its ring, and calls on other streams
-// run beside this one only if their blocks all fit.  One call, and 16 calls on
-// 16 streams, in ms, on the clusters and the wide mode / with tiles in all slots /
-// by this rule (u8): 512^2 at lambda = 0 0.56 / 0.22 / 0.22 and 1.54 / 2.95 /
-// 0.91, at lambda = 20 6.9 / 2.7 / 2.9 and 10.6 / 39.2 / 8.9; 256^2 3.1 / 1.4 /
-// 1.55 and 5.9 / 11.4 / 3.6; 1000^2 17.4 / 5.0 / 5.3 and 33.9 / 79.6 / 33.3;
-// 2048^2 at lambda = 30 30.0 / 11.7 / 13.2 and 173 / 188 / 122; 4 batches of 4
-// 512^2 images on 4 streams 10.3 / 13.8 / 7.8.  A tile every 8 or 12 pixels: one
-// call 4 % less or 6 % more, 16 at once 30 % more or 8 % less.  (Long strips need
-// more tiles than that: all slots.)
 bool mosaic_shape(const JobSpec *jobs, int n, MosaicShape *out)
 {
     const bool any16 = jobs[0].dtype == THIN_U16;
@@ -466,32 +448,7 @@ bool mosaic_shape(const JobSpec *jobs, int n, MosaicShape *out)
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-    const int limit = std::min(optin, per_sm / 2 - reserved) - 256;
-    const int slots = 2 * sms;
-    double want = 0;
-    for (int k = 0; k < n; ++k) want += std::max(std::sqrt(double(jobs[k].w) * jobs[k].h) / 10, 8.0);
-    for (int most : {slots / std::max(int(slots / want + 0.6), 1), slots}) {
-        // for every width the lowest tile that gives few enough tiles; of these the smallest with its halo
-        double best = 0;
-        for (int tw = 32; tw <= 224; tw += 16) {
-            int lo = 16, hi = 304;
-            if (mosaic_tiles(jobs, n, tw, hi) > most) continue;
-            while (lo < hi) {
-                const int mid = (lo + hi) / 16 * 8;  // a multiple of 8 below hi
-                if (mosaic_tiles(jobs, n, tw, mid) <= most) hi = mid;
-                else lo = mid + 8;
-            }
-            const double cost = double(tw + 16) * (hi + 16);
-            if ((best == 0 || cost < best) && tile_layout(tw, hi, halo_rows(kMaxStep), any16).bytes <= limit) {
-                best = cost;
-                out->tw = tw;
-                out->th = hi;
-                out->halo = kMaxStep;
-            }
-        }
-        if (best > 0) return true;
-    }
-    return false;
+    return mosaic_search(jobs, n, any16, sms, std::min(optin, per_sm / 2 - reserved) - 256, out);
 }
 
 int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const thin_options &opt, cudaStream_t stream,

@@ -8,51 +8,10 @@
 
 #include "thin_block.cuh"
 #include "thin_common.cuh"
+#include "thin_layout.h"
 #include "thin_simd.cuh"
 
 namespace thin {
-
-constexpr int kWarps = 8;
-constexpr int kThreads = 32 * kWarps;
-constexpr int kMinHalo = 3;
-constexpr int kPadCols = 16;   // halo columns staged on each side of a tile (two cells)
-constexpr int kMaxStep = 15;   // phases a step can have: one halo column more than that is needed
-
-// Shared memory of a block: decision table, control words, tile rows, dirty
-// bitmaps (a word per cell row and parity: a tile and its halo are at most 32
-// cells wide), queue of groups.
-struct TileLayout {
-    int row_bytes;   // bytes of a staged row (tile and halo columns)
-    int rows;        // staged rows
-    int box_rows;    // rows of one TMA box (one or two boxes to a tile)
-    int dirty_off, queue_off, bytes;
-};
-constexpr int kOffCtrl = (kDecisionBytes + 15) / 16 * 16;  // control words, then the mbarrier
-constexpr int kOffBar = kOffCtrl + 32;
-constexpr int kOffTile = (kOffBar + 8 + 127) / 128 * 128 + 128;  // TMA destinations are 128-byte aligned
-
-inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-
-// Shared memory of a block for tiles tw x th with hr halo rows.  A tile of more
-// than 256 staged rows takes two TMA boxes, each starting at a multiple of 128 bytes.
-inline TileLayout tile_layout(int tw, int th, int hr, bool any16)
-{
-    TileLayout L;
-    L.row_bytes = (tw + 2 * kPadCols) * (any16 ? 2 : 1);
-    L.rows = th + 2 * hr;
-    L.box_rows = L.rows;
-    if (L.rows > 256) {
-        L.box_rows = int(align_up(size_t(L.rows + 1) / 2, 8));
-        L.rows = 2 * L.box_rows;
-    }
-    L.dirty_off = int(align_up(size_t(kOffTile) + size_t(L.row_bytes) * L.rows + 16, 16));
-    L.queue_off = L.dirty_off + 4 * 4 * (L.rows / 2);
-    L.bytes = L.queue_off + 2 * 32 * (L.rows / 2);
-    return L;
-}
-
-// Halo rows for steps of H phases: one pixel more than phases, even.
-inline int halo_rows(int H) { return (H + 2) / 2 * 2; }
 
 __device__ __forceinline__ unsigned long long gtimer()
 {

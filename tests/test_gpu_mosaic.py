@@ -58,3 +58,36 @@ def test_set_tile_shape_is_still_checked():
     with pytest.raises(thin.ThinError):
         thin.batch(work, [60] * 3, halo=9)
     assert all(np.array_equal(t.cpu().numpy(), img) for t in work)
+
+
+def _naive(img, lam):
+    """The phases one launch after another, straight from global memory (no tiles)."""
+    t = torch.from_numpy(img).cuda()
+    st = thin.run(t, lam, kernel="naive")
+    return t, st
+
+
+@pytest.mark.parametrize("h,w,lams,n", [(1548, 1470, (0, 80), 1), (965, 693, (0, 80), 1), (794, 870, (40,), 1), (2000, 2000, (0,), 1),
+                                        (2048, 2048, (0, 30), 1), (1200, 1200, (30,), 4), (700, 700, (30,), 16)])
+def test_high_u16_tiles(h, w, lams, n):
+    """u16 images whose tiles are 200 to 300 rows high, several side by side."""
+    for lam in lams:
+        imgs = [synth.value_noise_image(h, w, "u16", seed=h + w + k) for k in range(min(n, 2))]
+        want = [_naive(im, lam) for im in imgs]
+        work = [torch.from_numpy(imgs[k % len(imgs)]).cuda() for k in range(n)]
+        stats, rc = thin.batch(work, [lam] * n)
+        assert rc == 0
+        for k, (t, st) in enumerate(zip(work, stats)):
+            ref, rst = want[k % len(imgs)]
+            assert st["tiles_visited"] == 0 and st["converged"] == 1
+            assert torch.equal(t.view(torch.int16), ref.view(torch.int16))
+            assert st["lowered"] == rst["lowered"] and st["last_change_phase"] == rst["last_change_phase"]
+
+
+def test_high_u16_tiles_against_the_oracle():
+    img = synth.value_noise_image(965, 693, "u16", seed=9)
+    ref, rst = oracle.thin(img, 0)
+    t = torch.from_numpy(img).cuda()
+    st = thin.run(t, 0)
+    assert np.array_equal(t.cpu().numpy(), ref)
+    assert st["lowered"] == rst["lowered"] and st["last_change_phase"] == rst["last_change_phase"]
