@@ -64,6 +64,19 @@ constexpr int kMosMaxRows = 304;  // the highest tile
 // from global memory, es 16-byte vectors a side and row: enough for the highest tile.
 constexpr int mosaic_side_turns(int es) { return (2 * es * kMosMaxRows + kThreads - 1) / kThreads; }
 
+// What the exchange of rims and the phases rest on (es: element size).
+constexpr bool mosaic_shape_fits(int es, const MosaicShape &s)
+{
+    const int hr = (s.halo + 2) / 2 * 2;  // halo_rows
+    return s.tw % 16 == 0 && s.th % 2 == 0 &&              // cells of 8 x 2, vectors of 16 bytes
+           s.halo >= 1 && s.halo < kPadCols &&             // a halo column more than a step has phases
+           s.tw >= kPadCols && s.th >= hr &&               // a halo reaches into the next tile only
+           s.tw / 8 + 4 <= 32 && s.tw * es / 16 + 2 * es <= 32 &&  // a lane to a cell, a lane to a vector of a row
+           hr <= 2 * kWarps &&                             // the halo's rows in four turns of the warps, its cell rows in two
+           s.th <= kMosMaxRows && 2 * es * s.th <= mosaic_side_turns(es) * kThreads &&  // the side columns
+           (s.th + 2 * hr + 16) / 2 <= kThreads;           // a thread to a cell row (two TMA boxes round the rows up)
+}
+
 template <typename Job>
 int mosaic_tiles(const Job *jobs, int n, int tw, int th)
 {

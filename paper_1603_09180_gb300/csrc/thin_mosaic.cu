@@ -461,6 +461,7 @@ int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const t
     for (int k = 1; k < n; ++k)
         if (elem_size(jobs[k].dtype) != M->es) return THIN_ERR_ARG;  // one element size per launch
     const bool any16 = M->es == 2;
+    if (!mosaic_shape_fits(M->es, shape)) return THIN_ERR_ARG;
     const int tw = shape.tw, th = shape.th, H = shape.halo;
     const TileLayout L = tile_layout(tw, th, halo_rows(H), any16);
     std::vector<MosImage> imgs(n);

@@ -2,7 +2,8 @@
 
 The choice is host arithmetic (csrc/thin_layout.h), so a host compiler can run it: every shape it
 returns, for one to 16 images of either type on GPUs of 152 and of 148 SMs, lies within the turns in
-which a block moves its rims' side columns (2 es 16-byte vectors a row, a thread to a vector)."""
+which a block moves its rims' side columns (2 es 16-byte vectors a row, a thread to a vector) and within
+the other bounds of the kernel, which a launch checks; shapes just past a bound are refused."""
 import math
 import os
 import random
@@ -29,7 +30,8 @@ int main()
             if (scanf("%d %d", &j.w, &j.h) != 2) return 1;
         thin::MosaicShape s = {0, 0, 0};
         const bool ok = thin::mosaic_search(jobs.data(), n, es == 2, sms, limit, &s);
-        printf("%d %d %d %d %d\n", int(ok), s.tw, s.th, s.halo, thin::mosaic_side_turns(es) * thin::kThreads);
+        printf("%d %d %d %d %d %d\n", int(ok), s.tw, s.th, s.halo, thin::mosaic_side_turns(es) * thin::kThreads,
+               int(thin::mosaic_shape_fits(es, s)));
     }
 }
 """
@@ -67,6 +69,22 @@ def calls(es, sms):
 @pytest.mark.parametrize("sms", [148, 152])
 def test_side_columns_of_every_shape_are_exchanged(search, es, sms):
     got = search(calls(es, sms))
-    tw, th, halo, vectors = got[got[:, 0] == 1][:, 1:].T
+    tw, th, halo, vectors, fits = got[got[:, 0] == 1][:, 1:].T
     assert len(tw) > 3000 and th.max() > 192
     assert (2 * es * th <= vectors).all()
+    assert fits.all()
+
+
+@pytest.mark.parametrize("es,tw,th,halo,ok", [
+    (1, 32, 16, 15, 1), (2, 32, 16, 15, 1), (1, 224, 304, 15, 1), (2, 224, 304, 15, 1), (1, 16, 16, 1, 1),
+    (1, 224, 306, 15, 0), (2, 32, 312, 15, 0), (1, 240, 64, 15, 0), (2, 240, 64, 15, 0), (1, 40, 64, 15, 0),
+    (1, 32, 15, 3, 0), (1, 32, 14, 15, 0), (1, 0, 64, 15, 0), (1, 32, 64, 16, 0), (1, 32, 64, 0, 0)])
+def test_bounds(tmp_path, es, tw, th, halo, ok):
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no host compiler")
+    (tmp_path / "b.cpp").write_text('#include "thin_layout.h"\n'
+                                    "static_assert(thin::mosaic_shape_fits(%d, thin::MosaicShape{%d, %d, %d}) == %s, \"\");\n"
+                                    % (es, tw, th, halo, "true" if ok else "false"))
+    subprocess.run([cxx, "-std=c++17", "-fsyntax-only", "-fconstexpr-ops-limit=200000000", "-I", CSRC, str(tmp_path / "b.cpp")],
+                   check=True)
