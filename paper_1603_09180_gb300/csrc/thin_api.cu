@@ -156,6 +156,7 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     G->wide.clear();
     G->mosaic.clear();
     G->tiled.clear();
+    G->tiled_fits.clear();
     // (a call that sets a tile shape has it checked where images go to the tiled engine: it keeps that route)
     const bool own_tiles = o.tile_w || o.tile_h || o.halo;
     if (allow_wide && o.kernel == THIN_KERNEL_AUTO && !own_tiles && n <= kMosaicMax &&
@@ -224,7 +225,10 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     for (int k = 0; k < n; ++k) {
         if (cls[k] > 0) continue;
         if (use_wide && strips[k] > 0) G->wide.push_back({k, strips[k], csize[k]});
-        else G->tiled.push_back(k);
+        else {
+            G->tiled.push_back(k);
+            G->tiled_fits.push_back(cls[k] < 0);
+        }
     }
     if (!G->tiled.empty() && o.kernel == THIN_KERNEL_RESIDENT) return THIN_ERR_ARG;  // does not fit on chip
     return THIN_OK;
@@ -302,7 +306,10 @@ int Execution::prepare(const std::vector<JobSpec> &specs_in, const Grouping &G, 
     }
     if (!G.tiled.empty()) {
         std::vector<JobSpec> js;
-        for (int k : G.tiled) js.push_back(specs[k]);
+        for (size_t i = 0; i < G.tiled.size(); ++i) {
+            js.push_back(specs[G.tiled[i]]);
+            js.back().fits_cluster = G.tiled_fits[i] != 0;
+        }
         tiled_idx = G.tiled;
         const int rc = tiled_prepare(js.data(), int(js.size()), o, s, async_alloc, &tiled, tiled_max_grid);
         if (rc != THIN_OK) return rc;

@@ -32,7 +32,18 @@ struct JobSpec {
     uint32_t lam;
     int adj;        // THIN_ADJ_8_4 / THIN_ADJ_4_8
     int done_slot = -1;  // resident engine: completion record to post when the image is finished, -1 none
+    bool fits_cluster = false;  // tiled engine: the image fits a cluster, so its stats keep the resident engine's rule at a cap
 };
+
+// The resident engine's rule at a phase cap: converged if the last three
+// phases changed nothing.  `last`: last phase that lowered a point, -1 if none.
+// Where a default call takes another engine for images that fit a cluster (or
+// the wide mode), its status at a cap stays what this rule says, whenever that
+// engine saw its fixed point.
+inline bool quiet_at_cap(const thin_options &o, long long last)
+{
+    return o.max_phases >= 4 && last < o.start_phase + o.max_phases - 3;
+}
 
 inline int elem_size(int dtype) { return dtype == THIN_U16 ? 2 : 1; }
 
@@ -232,6 +243,7 @@ struct Grouping {
     std::vector<int> mosaic;  // one launch
     MosaicShape mosaic_tile;
     std::vector<int> tiled;
+    std::vector<char> tiled_fits;  // per entry of tiled: it would fit a cluster
 };
 // allow_wide: large images may take the wide resident mode (a cooperative
 // launch over the whole GPU); serving turns it off so that its lanes share

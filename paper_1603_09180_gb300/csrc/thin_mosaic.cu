@@ -578,11 +578,13 @@ int mosaic_collect(const MosaicPrepared &M, const thin_options &opt, cudaStream_
         long long phases = S.stop ? (long long)S.stop * M.halo : opt.max_phases;
         if (opt.max_phases >= 0) phases = std::min<long long>(phases, opt.max_phases);
         if (phases < 0) phases = 0;  // (a run that ended with an error)
-        o.converged = S.stop != 0 && !error;
+        const long long last = (long long)S.last - 1;
+        o.converged = S.stop != 0 && !error && (opt.max_phases < 0 || quiet_at_cap(opt, last));
+        if (S.stop && !error && !o.converged) phases = opt.max_phases;  // (the phases after the stop change nothing)
         o.status = error ? error : (o.converged ? THIN_OK : THIN_ERR_NOT_CONVERGED);
         o.phases = phases;
         o.lowered = (int64_t)S.lowered;
-        o.last_change_phase = (int64_t)S.last - 1;
+        o.last_change_phase = last;
         o.end_phase = opt.start_phase + phases;
         o.steps = (phases + M.halo - 1) / M.halo;
         o.tested = (int64_t)S.tested;

@@ -770,6 +770,10 @@ int tiled_collect(const TiledPrepared *T, const thin_options &opt, cudaStream_t 
         long long phases = steps * T->H;
         if (opt.max_phases >= 0) phases = std::min<long long>(phases, opt.max_phases);
         o.converged = (S.last_listed <= S.last_step && ctl.error == 0) ? 1 : 0;
+        if (T->jobs[k].fits_cluster && opt.max_phases >= 0 && ctl.error == 0) {
+            o.converged = quiet_at_cap(opt, S.last_change);
+            if (!o.converged) phases = opt.max_phases;
+        }
         o.status = ctl.error ? ctl.error : (o.converged ? THIN_OK : THIN_ERR_NOT_CONVERGED);
         o.phases = phases;
         o.lowered = (int64_t)S.lowered;
