@@ -11,11 +11,9 @@
 
 #include "thin_common.cuh"
 #include "thin_internal.h"
+#include "thin_pool.h"
 
 namespace thin {
-
-typedef CUresult (*CtxGetCurrentFn)(CUcontext *);
-typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long *);
 
 int cuda_status(cudaError_t e)
 {
@@ -24,37 +22,78 @@ int cuda_status(cudaError_t e)
     return e == cudaErrorMemoryAllocation ? THIN_ERR_OOM : THIN_ERR_CUDA;
 }
 
+namespace {
+
+// The driver functions that tell contexts apart; null where the driver lacks one.
+struct DriverFns {
+    CUresult (*ctx_get_current)(CUcontext *) = nullptr;
+    CUresult (*ctx_get_id)(CUcontext, unsigned long long *) = nullptr;
+    CUresult (*device_get)(CUdevice *, int) = nullptr;
+    CUresult (*primary_get_state)(CUdevice, unsigned *, int *) = nullptr;
+    CUresult (*primary_retain)(CUcontext *, CUdevice) = nullptr;
+    CUresult (*primary_release)(CUdevice) = nullptr;
+};
+
+template <typename Fn>
+void driver_fn(const char *name, Fn *fn)
+{
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+        *fn = reinterpret_cast<Fn>(p);
+}
+
+const DriverFns &driver()
+{
+    static DriverFns D;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        driver_fn("cuCtxGetCurrent", &D.ctx_get_current);
+        driver_fn("cuCtxGetId", &D.ctx_get_id);
+        driver_fn("cuDeviceGet", &D.device_get);
+        driver_fn("cuDevicePrimaryCtxGetState", &D.primary_get_state);
+        driver_fn("cuDevicePrimaryCtxRetain", &D.primary_retain);
+        driver_fn("cuDevicePrimaryCtxRelease", &D.primary_release);
+    });
+    return D;
+}
+
+// Whether the calling thread's current context is the primary one of device `dev`.
+bool primary_is_current(int dev)
+{
+    const DriverFns &D = driver();
+    if (!D.ctx_get_current || !D.device_get || !D.primary_get_state || !D.primary_retain || !D.primary_release) return false;
+    CUcontext c = nullptr, p = nullptr;
+    CUdevice d = 0;
+    unsigned flags = 0;
+    int active = 0;
+    if (D.ctx_get_current(&c) != CUDA_SUCCESS || !c || D.device_get(&d, dev) != CUDA_SUCCESS) return false;
+    if (D.primary_get_state(d, &flags, &active) != CUDA_SUCCESS || !active) return false;  // (not created for the question's sake)
+    if (D.primary_retain(&p, d) != CUDA_SUCCESS) return false;
+    D.primary_release(d);
+    return c == p;
+}
+
+}  // namespace
+
 // Identity of the calling thread's current context, 0 if it cannot be had.
 unsigned long long current_context_id()
 {
-    static CtxGetCurrentFn get_current = nullptr;
-    static CtxGetIdFn get_id = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_current = reinterpret_cast<CtxGetCurrentFn>(p);
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_id = reinterpret_cast<CtxGetIdFn>(p);
-    });
+    const DriverFns &D = driver();
     CUcontext c = nullptr;
     unsigned long long id = 0;
-    if (get_current && get_id && get_current(&c) == CUDA_SUCCESS && c && get_id(c, &id) == CUDA_SUCCESS) return id;
+    if (D.ctx_get_current && D.ctx_get_id && D.ctx_get_current(&c) == CUDA_SUCCESS && c &&
+        D.ctx_get_id(c, &id) == CUDA_SUCCESS)
+        return id;
     return 0;
 }
 
 namespace {
 
 // The library's memory pools, one per device.
-struct ScratchPool {
-    unsigned long long ctx_id = 0;  // context the pool belongs to
-    cudaMemPool_t pool = nullptr;
-};
 std::mutex g_scratch_mu;
-ScratchPool g_scratch[64];
+PoolSlot<cudaMemPool_t> g_scratch[64];
 constexpr unsigned long long kScratchKeep = 256ull << 20;
 
 cudaMemPool_t scratch_pool()
@@ -62,24 +101,20 @@ cudaMemPool_t scratch_pool()
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
     std::lock_guard<std::mutex> lock(g_scratch_mu);
-    ScratchPool &S = g_scratch[dev];
-    const unsigned long long id = current_context_id();
-    if (id == 0) return nullptr;
-    if (!S.pool || S.ctx_id != id) {  // (a context created anew has lost the old pool)
-        cudaMemPoolProps props;
-        std::memset(&props, 0, sizeof props);
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t pool = nullptr;
-        unsigned long long keep = kScratchKeep;
-        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
-            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess)
-            return nullptr;
-        S.pool = pool;
-        S.ctx_id = id;
-    }
-    return S.pool;
+    return pool_for(
+        g_scratch[dev], current_context_id(), [&] { return primary_is_current(dev); },
+        [&](cudaMemPool_t *pool) {
+            cudaMemPoolProps props;
+            std::memset(&props, 0, sizeof props);
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            unsigned long long keep = kScratchKeep;
+            if (cudaMemPoolCreate(pool, &props) != cudaSuccess) return false;
+            if (cudaMemPoolSetAttribute(*pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) return true;
+            cudaMemPoolDestroy(*pool);
+            return false;
+        });
 }
 
 }  // namespace
