@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 from dataclasses import dataclass
 
 import numpy as np
@@ -302,22 +303,35 @@ class Server:
         if rc != THIN_OK:
             raise ThinError(rc, "thin_serve_create")
         self.shapes = {}
+        self._known = threading.Condition()
+        self._submitting = 0  # submits whose ticket may be out, and finished, before `shapes` holds it
 
     def submit(self, img: np.ndarray, lam: int) -> int:
         if img.ndim != 2 or img.dtype not in (np.uint8, np.uint16) or (img.size and img.strides[1] != img.itemsize):
             raise ValueError("image must be a 2-D uint8/uint16 array with unit column stride")
         h, w = img.shape
         t = ctypes.c_uint64()
-        rc = self._lib.thin_serve_submit(self._h, ctypes.c_void_p(img.ctypes.data if img.size else 0), w, h,
-                                         img.strides[0] if h > 1 else w * img.itemsize,
-                                         U16 if img.dtype == np.uint16 else U8, int(lam), ctypes.byref(t))
+        with self._known:
+            self._submitting += 1
+        try:
+            rc = self._lib.thin_serve_submit(self._h, ctypes.c_void_p(img.ctypes.data if img.size else 0), w, h,
+                                             img.strides[0] if h > 1 else w * img.itemsize,
+                                             U16 if img.dtype == np.uint16 else U8, int(lam), ctypes.byref(t))
+        finally:
+            with self._known:
+                if t.value:
+                    self.shapes[t.value] = (h, w, img.dtype)
+                self._submitting -= 1
+                self._known.notify_all()
         if rc != THIN_OK:
             raise ThinError(rc, "thin_serve_submit")
-        self.shapes[t.value] = (h, w, img.dtype)
         return t.value
 
     def poll(self, ticket: int):
         """(done, result array or None, stats dict or None, rc)."""
+        if ticket not in self.shapes:  # another thread's submit may not have returned yet
+            with self._known:
+                self._known.wait_for(lambda: ticket in self.shapes or self._submitting == 0)
         h, w, dt = self.shapes[ticket]
         out = np.empty((h, w), dt)
         done = ctypes.c_int()
