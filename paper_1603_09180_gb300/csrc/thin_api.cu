@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -127,6 +128,8 @@ cudaMemPool_t scratch_pool()
 // gives memory back in the same way, and all of it if an allocation fails.
 cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t stream)
 {
+    if (const char *most = std::getenv("THIN_SCRATCH_MAX"))  // (for tests: scratch that runs out)
+        if (bytes > std::strtoull(most, nullptr, 10)) return cudaErrorMemoryAllocation;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaMemPool_t pool = nullptr;
     if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) pool = scratch_pool();
@@ -184,7 +187,7 @@ int check_image(const void *img, int w, int h, size_t pitch, int dt)
 // the tiled engine (AUTO, TILED).  When few images fit, each is spread over a
 // wider cluster (at least 32 rows a block) so that more SMs work on it.
 constexpr int kWideMax = 2;
-int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Grouping *G, bool allow_wide)
+int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Grouping *G, bool allow_wide, bool spare)
 {
     const int n = int(specs.size());
     G->resident.clear();
@@ -194,7 +197,7 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     G->tiled_fits.clear();
     // (a call that sets a tile shape has it checked where images go to the tiled engine: it keeps that route)
     const bool own_tiles = o.tile_w || o.tile_h || o.halo;
-    if (allow_wide && o.kernel == THIN_KERNEL_AUTO && !own_tiles && n <= kMosaicMax &&
+    if (allow_wide && !spare && o.kernel == THIN_KERNEL_AUTO && !own_tiles && n <= kMosaicMax &&
         mosaic_shape(specs.data(), n, &G->mosaic_tile)) {
         for (int k = 0; k < n; ++k) G->mosaic.push_back(k);
         return THIN_OK;
@@ -216,7 +219,7 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
     // resident 262 / 221 / 202 ms.  (Serving, which passes allow_wide = false,
     // keeps them resident: its small lanes retire image by image.  So does a call
     // that sets a tile shape, which not every image may take.)
-    if (allow_wide && o.kernel == THIN_KERNEL_AUTO && !own_tiles) {
+    if (allow_wide && !spare && o.kernel == THIN_KERNEL_AUTO && !own_tiles) {
         int count[17] = {};
         for (int k = 0; k < n; ++k) ++count[cls[k]];
         const int huge = count[0] > kWideMax ? count[0] : 0;
@@ -352,6 +355,17 @@ int Execution::prepare(const std::vector<JobSpec> &specs_in, const Grouping &G, 
     return THIN_OK;
 }
 
+int Execution::prepare_or_spare(const std::vector<JobSpec> &specs_in, Grouping *G, const thin_options &group,
+                                const thin_options &o, cudaStream_t s)
+{
+    int rc = prepare(specs_in, *G, o, s, true);
+    if (rc != THIN_ERR_OOM || !G->can_spare()) return rc;
+    release(s);
+    *this = Execution();
+    rc = group_jobs(specs_in, group, G, true, true);
+    return rc == THIN_OK ? prepare(specs_in, *G, o, s, true) : rc;
+}
+
 // Resident groups run side by side on helper streams forked from s (a
 // group's clusters take SMs as another group's finish); the wide launches and
 // the tiled group, whose grid barriers need all their blocks resident at
@@ -422,8 +436,7 @@ namespace {
 
 // Runs validated images in one device-driven pass: every launch group
 // prepared, enqueued side by side, stats collected if asked for.
-int dispatch(const std::vector<JobSpec> &specs, const thin_options &o, cudaStream_t s, thin_stats *out,
-             bool allow_wide = true)
+int dispatch(const std::vector<JobSpec> &specs, const thin_options &o, cudaStream_t s, thin_stats *out)
 {
     if (o.max_phases == 0) {  // nothing may run: every image stays as it is, unconverged
         if (out)
@@ -436,15 +449,15 @@ int dispatch(const std::vector<JobSpec> &specs, const thin_options &o, cudaStrea
         return THIN_ERR_NOT_CONVERGED;
     }
     Grouping G;
-    int rc = group_jobs(specs, o, &G, allow_wide);
+    int rc = group_jobs(specs, o, &G);
     if (rc != THIN_OK) return rc;
-    SideStreams *ss = nullptr;
-    if (G.resident.size() > 1) {
-        const cudaError_t e = side_streams(&ss);
-        if (e != cudaSuccess) return cuda_status(e);
-    }
     Execution X;
-    rc = X.prepare(specs, G, o, s, true);
+    rc = X.prepare_or_spare(specs, &G, o, o, s);
+    SideStreams *ss = nullptr;
+    if (rc == THIN_OK && G.resident.size() > 1) {
+        const cudaError_t e = side_streams(&ss);
+        if (e != cudaSuccess) rc = cuda_status(e);
+    }
     if (rc == THIN_OK) {
         const cudaError_t e = X.enqueue(s, ss ? ss->s : nullptr, ss ? ss->ev : nullptr);
         if (e != cudaSuccess) rc = cuda_status(e);

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <vector>
 
@@ -244,11 +245,16 @@ struct Grouping {
     MosaicShape mosaic_tile;
     std::vector<int> tiled;
     std::vector<char> tiled_fits;  // per entry of tiled: it would fit a cluster
+    // a grouping made with `spare` needs less scratch
+    bool can_spare() const { return !mosaic.empty() || std::count(tiled_fits.begin(), tiled_fits.end(), 1) > 0; }
 };
 // allow_wide: large images may take the wide resident mode (a cooperative
 // launch over the whole GPU); serving turns it off so that its lanes share
-// the GPU.
-int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Grouping *G, bool allow_wide = true);
+// the GPU.  spare: images that fit a cluster or the wide mode stay there, which
+// need next to no scratch (the mosaic engine takes twice the images' size and
+// the tiled engine once).
+int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Grouping *G, bool allow_wide = true,
+               bool spare = false);
 
 // Every launch group of a batch, prepared; enqueue() is device work only
 // (resident groups forked onto up to four side streams with events, joined
@@ -269,6 +275,10 @@ struct Execution {
     std::vector<int> tiled_idx;
     int prepare(const std::vector<JobSpec> &specs, const Grouping &G, const thin_options &o, cudaStream_t s,
                 bool async_alloc);
+    // prepare with stream-ordered scratch; where that runs out, once more by the grouping of options `group`
+    // that spares it (G is replaced).
+    int prepare_or_spare(const std::vector<JobSpec> &specs, Grouping *G, const thin_options &group, const thin_options &o,
+                         cudaStream_t s);
     cudaError_t enqueue(cudaStream_t s, cudaStream_t *side, cudaEvent_t *ev) const;
     int collect(cudaStream_t s, thin_stats *out) const;  // out[k] for specs[k]; waits for s
     void release(cudaStream_t s);

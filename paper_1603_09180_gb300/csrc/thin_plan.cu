@@ -134,7 +134,8 @@ int thin_plan_create(const thin_job *jobs, int n, thin_adj adj, const thin_optio
         p->halo = ot.tile_w ? ot.halo : fill_halo;
     }
     if (e == cudaSuccess) {
-        rc = p->X.prepare(p->specs, G, ot, cs, true);  // plan-owned device memory, stream-ordered on cs
+        rc = p->X.prepare_or_spare(p->specs, &G, o, ot, cs);  // plan-owned device memory, stream-ordered on cs
+        if (G.tiled.empty()) p->tile_w = p->tile_h = p->halo = 0;
         if (rc == THIN_OK) e = cudaStreamSynchronize(cs);  // tables uploaded before capture
         if (rc == THIN_OK && e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         if (rc == THIN_OK && e == cudaSuccess) {
