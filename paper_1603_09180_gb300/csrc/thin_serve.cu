@@ -141,6 +141,7 @@ struct thin_server {
     size_t used = 0;   // bytes charged by admitted requests
     int in_flight = 0;
     bool stop = false;
+    int ready = 0;     // lanes that have set themselves up
     uint64_t next_ticket = 1;
     std::vector<std::thread> lanes;
     thin::PinnedArena pool;
@@ -200,6 +201,11 @@ void lane_main(thin_server *S)
         cudaGetLastError();
         ok_lane = false;
     }
+    {
+        std::lock_guard<std::mutex> g(S->mu);
+        ++S->ready;
+    }
+    S->cv.notify_all();
     // a large batch's tiled launch takes at most a quarter of the SMs (two may run), so that
     // the resident launches of the other lanes keep running beside them: two blocks to an SM
     // (48 requests of every size: 63 ms with one, 46 with two, 49 with three)
@@ -396,6 +402,12 @@ int thin_serve_create(size_t device_budget_bytes, int max_slots, int queue_cap, 
         return THIN_ERR_OOM;
     }
     for (int k = 0; k < kLanes; ++k) S->lanes.emplace_back(lane_main, S);
+    // A lane's set-up (pinned memory, streams) waits for running kernels to end and holds up the other
+    // lanes' calls meanwhile, result copies too: no request is taken before every lane has done with it.
+    {
+        std::unique_lock<std::mutex> g(S->mu);
+        S->cv.wait(g, [&] { return S->ready == kLanes; });
+    }
     *out = S;
     return THIN_OK;
 }

@@ -167,3 +167,19 @@ def test_serve_budget_admits_one_at_a_time():
             ref, _ = alone(imgs[tickets.index(t)], 5)
             assert np.array_equal(out, ref)
     assert order == tickets  # one admitted at a time, first come first served
+
+
+def test_first_requests_of_a_server_do_not_wait_for_a_slow_one():
+    """As above, on twelve servers in turn, each asked right after it was made."""
+    slow = synth.value_noise_image(512, 512, "u8", seed=38)
+    small = [synth.value_noise_image(48, 64, "u8", seed=100 + k) for k in range(40)]
+    for _ in range(12):
+        with thin.Server(1 << 30, max_slots=8 * 64, queue_cap=64) as srv:
+            ts = srv.submit(slow, 20)
+            left = {srv.submit(im, 0) for im in small} | {ts}
+            while left:
+                t = srv.wait_any(20000)
+                assert t is not None
+                left.discard(t)
+                srv.poll(t)
+                assert t != ts or not left
