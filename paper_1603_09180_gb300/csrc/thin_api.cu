@@ -275,20 +275,21 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
 namespace {
 
 // Helper streams of the calling host thread for running launch groups side
-// by side (created once per thread and device, kept until the process exits).
+// by side (created once per thread and device, kept until the process exits or
+// the thread gives them back).
 struct SideStreams {
     int dev = -1;
     cudaStream_t s[kMaxResidentGroups] = {};
     cudaEvent_t ev[kMaxResidentGroups + 1] = {};
 };
+thread_local SideStreams t_side;
 
 cudaError_t side_streams(SideStreams **out)
 {
-    thread_local SideStreams t;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (t.dev != dev) {
+    if (t_side.dev != dev) {
         SideStreams n;
         n.dev = dev;
         for (auto &x : n.s)
@@ -296,9 +297,9 @@ cudaError_t side_streams(SideStreams **out)
         for (auto &x : n.ev)
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
         if (e != cudaSuccess) return e;
-        t = n;
+        t_side = n;
     }
-    *out = &t;
+    *out = &t_side;
     return cudaSuccess;
 }
 
@@ -312,6 +313,15 @@ cudaError_t thread_side_streams(cudaStream_t **side, cudaEvent_t **ev)
     *side = ss->s;
     *ev = ss->ev;
     return cudaSuccess;
+}
+
+void release_thread_side_streams()
+{
+    for (auto x : t_side.s)
+        if (x) cudaStreamDestroy(x);
+    for (auto x : t_side.ev)
+        if (x) cudaEventDestroy(x);
+    t_side = SideStreams();
 }
 
 int Execution::prepare(const std::vector<JobSpec> &specs_in, const Grouping &G, const thin_options &o,

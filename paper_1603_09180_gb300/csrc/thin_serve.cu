@@ -369,6 +369,7 @@ void lane_main(thin_server *S)
     if (done_host) cudaFreeHost(done_host);
     if (copy) cudaStreamDestroy(copy);
     if (stream) cudaStreamDestroy(stream);
+    release_thread_side_streams();
 }
 
 }  // namespace

@@ -183,3 +183,15 @@ def test_first_requests_of_a_server_do_not_wait_for_a_slow_one():
                 left.discard(t)
                 srv.poll(t)
                 assert t != ts or not left
+
+
+def test_servers_give_their_device_memory_back():
+    """A server's streams go with it: the device's free memory after many servers is what it was after two."""
+    img = synth.value_noise_image(100, 120, "u8", seed=1)
+    free = []
+    for _ in range(12):
+        with thin.Server(1 << 28, max_slots=64, queue_cap=64) as srv:
+            k = srv.submit(img, 3)
+            collect(srv, 1)
+        free.append(torch.cuda.mem_get_info()[0])
+    assert free[1] - free[-1] < 64 << 20, [f >> 20 for f in free]  # (it lost 52 MiB a server)
