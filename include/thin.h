@@ -311,8 +311,11 @@ const char *thin_version(void);
  * An idle lane admits requests of one queue in arrival order while the slot
  * count and the byte budget allow, at most max_slots / 8 of them (a request
  * that does not fit waits at the head of its queue); at most two lanes at a
- * time take from the large queue, and each of their tiled launches uses at
- * most a quarter of the SMs, so small requests keep running beside them.
+ * time take from the large queue.  Each of their tiled launches has at most
+ * half as many blocks as the GPU has SMs.  Two can share an SM, so a launch
+ * starts once a quarter of the SMs are free, but where more are free it
+ * spreads over half of them: two such launches can hold every SM, and small
+ * requests then wait until one of them ends.
  * The lane allocates the device images, copies them in and launches them as
  * one batch (never the wide mode or the mosaic engine, so that the lanes
  * share the GPU).  Each

@@ -12,12 +12,12 @@
 // of the batch still runs, so queued requests are admitted by the next idle
 // lane as slots and memory free up.  Images too large for a cluster wait in
 // a queue of their own; at most two lanes at a time run a batch of them on
-// the tiled engine, each on at most a quarter of the SMs, and they retire
-// when their batch ends.  So small requests keep flowing on the other SMs
-// while large ones run.  (The tiled launch is cooperative: it starts only
-// when all its blocks fit at once.  Capped at half of the SMs it waited for
-// the long resident jobs to drain, and the small launches queued behind it;
-// two quarter-size launches start sooner and keep the same share.)
+// the tiled engine, and they retire when their batch ends.  A tiled launch has
+// at most half as many blocks as there are SMs.  It is cooperative: it starts
+// when all its blocks fit at once, which they do on a quarter of the SMs, two
+// to each; where more are free they spread, one to an SM (counted: 76 blocks
+// on 76 of 152 SMs, two launches at once on all 152).  So small requests keep
+// flowing beside one large batch, and may wait for one of two to end.
 // Lanes run side by side on the device (the resident engine gives each image
 // its own cluster and takes only the SMs it needs).  Each image's result depends
 // only on the image and its lambda: it is the same alone and in any mix.
@@ -206,9 +206,11 @@ void lane_main(thin_server *S)
         ++S->ready;
     }
     S->cv.notify_all();
-    // a large batch's tiled launch takes at most a quarter of the SMs (two may run), so that
-    // the resident launches of the other lanes keep running beside them: two blocks to an SM
-    // (48 requests of every size: 63 ms with one, 46 with two, 49 with three)
+    // The cap on a large batch's tiled launch, in blocks.  48 requests of every size take 63 ms with 38,
+    // 46 with 76 and 49 with 114.  Poisson arrivals of the same mix at 200 / 300 / 450 requests a second,
+    // medians of three seeds: with 38 blocks small images wait 1.3 / 1.4 / 2.3 ms (p90 15 / 27 / 50) and
+    // large ones 5.0 / 38 / 68 ms, and the mix queued at once runs at 450 images/s; with 76 small ones
+    // 1.6 / 2.7 / 12 ms (p90 37 / 51 / 70), large ones 2.5 / 4.1 / 30 ms, 800 images/s.
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, S->device);
     const int tiled_cap = std::max(1, 2 * (sms / (2 * kLargeLanes)));
