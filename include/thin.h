@@ -32,7 +32,12 @@
  * (a cudaStream_t passed as void*; NULL = the legacy default stream) unless a
  * stats pointer is given: then the call waits for the stream and fills the
  * stats before returning.  Scratch memory is taken from, and returned to,
- * the CUDA stream-ordered allocator on the same stream.
+ * the CUDA stream-ordered allocator on the same stream: from a memory pool of
+ * the library's own, one per device, which keeps up to 256 MiB of freed scratch
+ * for later calls until the device's context ends (or an allocation of the
+ * library's fails, which gives it all back).  Other allocators in the process
+ * have that much less.  Calls in a context other than the device's primary one
+ * use the device's default pool.
  *
  * Errors: every entry point returns THIN_OK (0) or a negative THIN_ERR_* code
  * and leaves the image untouched when it rejects its arguments.  Errors found
@@ -124,16 +129,21 @@ typedef struct {
 
 typedef struct {
     int32_t status;            /* THIN_OK, THIN_ERR_NOT_CONVERGED or THIN_ERR_TIMEOUT */
-    int32_t converged;         /* 1 if a quiet stretch of four phases was seen */
+    int32_t converged;         /* 1 if the image is at the schedule's fixed point.  At a phase cap the resident
+                                  engine, and AUTO for images that it or the mosaic engine takes, say so if the
+                                  last three phases changed nothing, the tiled engine after a step without a
+                                  change, the naive engine after a round of four phases without one */
     int64_t phases;            /* phases run by this call */
     int64_t lowered;           /* lowering steps F(x) := alpha^- performed */
     int64_t last_change_phase; /* global index of the last phase that lowered a point; -1 if none */
     int64_t end_phase;         /* global phase index to resume from */
     int64_t tiles_visited;     /* tile visits of the tiled kernel (0 for NAIVE) */
-    int64_t steps;             /* tile steps (tiled) or rounds of four phases (naive) */
+    int64_t steps;             /* tile steps (tiled, mosaic: of 15 phases each by default), phases (resident)
+                                  or rounds of four phases (naive) */
     int64_t tested;            /* point tests made: a point is tested in a phase of its parity only
                                   if a neighbour moved since its last test (all points in the first
-                                  four phases); the work behind the sweep rate */
+                                  four phases); the tiled engine tests some points once more when a
+                                  tile that rested is visited again; the work behind the sweep rate */
 } thin_stats;
 
 /* Fills *opt with the defaults (rule MAX, AUTO kernel, default tiles, phase 0, no cap, lambda-thinning). */

@@ -192,9 +192,9 @@ void tiled_release(TiledPrepared *T, cudaStream_t stream);
 // enough for its large tiles to fill the GPU (nothing to tune then).
 bool tiled_fills(const JobSpec *jobs, int n, int *tw, int *th, int *H);
 
-// Defaults of the tiled engine for a dtype (tile width/height in pixels, halo)
+// Defaults of the tiled engine (tile width/height in pixels, halo)
 // where the caller sets only some of them.
-void tiled_defaults(int dtype, int *tw, int *th, int *halo);
+void tiled_defaults(int *tw, int *th, int *halo);
 
 // Mosaic engine (thin_mosaic.cu): a few images whose tiles all fit in shared
 // memory at once, one block to a tile.
@@ -257,8 +257,8 @@ int group_jobs(const std::vector<JobSpec> &specs, const thin_options &o, Groupin
                bool spare = false);
 
 // Every launch group of a batch, prepared; enqueue() is device work only
-// (resident groups forked onto up to four side streams with events, joined
-// back before the tiled group), so it can be captured in a CUDA graph.
+// (resident groups forked onto up to kMaxResidentGroups side streams with
+// events, joined back before the others), so it can be captured in a CUDA graph.
 struct Execution {
     std::vector<JobSpec> specs;
     thin_options opt;

@@ -55,7 +55,7 @@ struct MosImage {
     unsigned long long rim[2];      // published pixels, laid out as the image
     unsigned long long rim_pitch;   // a multiple of 16
     unsigned long long bits[2];     // published dirty bits: a byte per cell, bit p for parity p
-    int w, h, dtype, adj;
+    int w, h, adj;
     unsigned lam;
     int tiles_x, tiles_y, tile_base;
     int cells_x;                    // cells of a row of `bits`
@@ -483,7 +483,6 @@ int mosaic_prepare(const JobSpec *jobs, int n, const MosaicShape &shape, const t
         I.pitch = J.pitch;
         I.w = J.w;
         I.h = J.h;
-        I.dtype = J.dtype;
         I.adj = J.adj;
         I.lam = J.lam;
         I.tiles_x = (J.w + tw - 1) / tw;

@@ -2,11 +2,11 @@
 // in shared memory for its whole run.
 //
 // Layout.  Block r of a cluster of C blocks holds image rows [r R, r R + R)
-// plus 8 halo rows of each neighbouring block, 16-byte padded.  A block runs 8
-// phases on its own (the exact region shrinks by one row per phase into the
-// halo), then copies fresh halo rows, and their dirty bits, from its
-// neighbours' shared memory (distributed shared memory) between two cluster
-// barriers.  A phase writes only points of its own parity and reads only the
+// plus 8 halo rows of each neighbouring block, or 16 where it has at least 64
+// rows of its own and the memory, 16-byte padded.  A block runs as many phases
+// on its own (the exact region shrinks by one row per phase into the halo),
+// then copies fresh halo rows, and their dirty bits, from its neighbours'
+// shared memory (distributed shared memory) between two cluster barriers.  A phase writes only points of its own parity and reads only the
 // other parities, so the blocks of a cluster never race inside a phase.
 // Clusters take images from a device-wide counter, longest first, so images
 // of different lengths run side by side without grid-wide synchronisation.

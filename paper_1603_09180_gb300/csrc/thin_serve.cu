@@ -156,7 +156,7 @@ size_t charge_of(int w, int h, int dtype, size_t *dpitch)
     *dpitch = (row + 15) / 16 * 16;
     const size_t img = *dpitch * size_t(h);
     // the image itself, plus the tiled engine's scratch for images too large
-    // for one cluster (a second buffer and 4 bytes per 8 x 2 cell), plus job
+    // for one cluster (a second buffer and 2 bytes per 8 x 2 cell), plus job
     // tables
     return img + img + size_t(w) * h / 4 + (64 << 10);
 }

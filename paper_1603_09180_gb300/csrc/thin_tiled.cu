@@ -12,8 +12,10 @@
 // parity a dirty bit per 4-point group, set by the moves of its neighbours that
 // can change its test, consumed by its phase.  Between visits the bits of an
 // image lie in global memory, a byte per cell with a bit per parity, in a
-// ping-pong pair of their own: a visit reads the bits of its tile and halo as
-// they were at the start of the step and writes those of its tile.  The halo is
+// ping-pong pair of their own: a visit reads the bits of its tile and halo from
+// one buffer and writes those of its tile to the other.  A tile that no step
+// visits keeps, in the buffer it was last read from, bits that its last visit
+// consumed: they add tests of points that cannot move and change nothing.  The halo is
 // one pixel wider than the step has phases, so that in the last phase too the
 // points just outside the tile are exact: every mark a neighbour's move makes
 // inside the tile is made by the tile's own visit, and no visit writes another
@@ -82,7 +84,7 @@ struct Ctl {
     int error;
     int steps;
     unsigned list_count[3];
-    unsigned next_item[3];  // per step (mod 3): items claimed beyond the first one of every warp
+    unsigned next_item[3];  // per step (mod 3): items claimed beyond the first one of every block
 };
 
 struct EngineArgs {
@@ -480,7 +482,7 @@ const EngineBuild &engine_build(int tiles, const TileLayout &L, int smem, int sm
 int tiled_shape(const JobSpec *jobs, int n, bool any16, const thin_options &opt, int *tw, int *th, int *H)
 {
     if (opt.tile_w || opt.tile_h || opt.halo) {
-        tiled_defaults(any16 ? THIN_U16 : THIN_U8, tw, th, H);
+        tiled_defaults(tw, th, H);
         if (opt.tile_w) *tw = opt.tile_w;
         if (opt.tile_h) *th = opt.tile_h;
         if (opt.halo) *H = opt.halo;
@@ -520,11 +522,11 @@ bool tiled_fills(const JobSpec *jobs, int n, int *tw, int *th, int *H)
     return *H == kMaxStep;  // (the large shapes)
 }
 
-void tiled_defaults(int dtype, int *tw, int *th, int *halo)
+void tiled_defaults(int *tw, int *th, int *halo)
 {
     *tw = 64;
     *th = 32;
-    *halo = dtype == THIN_U16 ? 8 : 8;
+    *halo = 8;
 }
 
 // A tiled launch prepared on the host: layout, tensor maps and pristine
@@ -831,7 +833,7 @@ int tiled_run(const JobSpec *jobs, int n, const thin_options &opt, cudaStream_t 
 // loop with a fixed time budget that may not call into the allocator, which
 // can have to map new memory or wait for the device.  thin_run_noalloc serves
 // them with the tiled engine and no allocation at all: its scratch (the
-// second ping-pong buffer, the change stamps, the worklists and the control
+// second ping-pong buffer, the dirty bits, the worklists and the control
 // words) lives in one fixed array in device memory that the library declares
 // at file scope.  Every GPU that loads the library holds the array until the
 // process exits.
