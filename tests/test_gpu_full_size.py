@@ -108,6 +108,16 @@ def test_large(name, kernel):
     torch.cuda.empty_cache()
 
 
+@pytest.mark.parametrize("name", ["large_4096_u8_s1603_l0", "large_4096_u8_s1603_l30"])
+def test_large_wide(name):
+    """4096^2 u8 in the wide resident mode, which the default call leaves to the mosaic engine."""
+    img = generate([name])[0]
+    t = to_dev(img)
+    st = thin.run(t, CASES[name]["lam"], kernel="resident")
+    assert st["tiles_visited"] == 0
+    expect(name, img, to_host(t), st)
+
+
 @pytest.mark.parametrize("runner", ["batch", "graph"])
 def test_uneven_1024(runner):
     """The 1024 uneven u8 images (sides 64..2048, lambda {0, 10, 25}) in one call: a thin_batch call,
