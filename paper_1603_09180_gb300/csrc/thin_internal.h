@@ -43,7 +43,7 @@ struct JobSpec {
 // engine saw its fixed point.
 inline bool quiet_at_cap(const thin_options &o, long long last)
 {
-    return o.max_phases >= 4 && last < o.start_phase + o.max_phases - 3;
+    return o.max_phases >= 4 && last - o.start_phase < o.max_phases - 3;  // (in this order nothing overflows)
 }
 
 inline int elem_size(int dtype) { return dtype == THIN_U16 ? 2 : 1; }

@@ -36,6 +36,15 @@ def test_one_image(img, lam, start):
             assert got["end_phase"] == start + cap
 
 
+@pytest.mark.parametrize("cap", [1 << 40, (1 << 63) - 1])
+def test_caps_out_of_reach(cap):
+    img = synth.value_noise_image(64, 64, "u8", seed=0)
+    full = thin.run(torch.from_numpy(img).cuda(), 10, start_phase=5)
+    for kernel in ("auto", "resident"):
+        st = thin.run(torch.from_numpy(img).cuda(), 10, start_phase=5, max_phases=cap, check=False, kernel=kernel)
+        assert [st[f] for f in FIELDS] == [full[f] for f in FIELDS]
+
+
 def test_batch_that_goes_to_tiles():
     img = torch.from_numpy(synth.value_noise_image(1300, 1310, "u8", seed=1)).cuda()
     last = thin.run(img.clone(), 0, kernel="resident")["last_change_phase"]
