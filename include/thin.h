@@ -138,7 +138,7 @@ typedef struct {
     int64_t last_change_phase; /* global index of the last phase that lowered a point; -1 if none */
     int64_t end_phase;         /* global phase index to resume from */
     int64_t tiles_visited;     /* tile visits of the tiled kernel (0 for NAIVE) */
-    int64_t steps;             /* tile steps (tiled, mosaic: of 15 phases each by default), phases (resident)
+    int64_t steps;             /* steps of up to 15 phases between exchanges (tiled, mosaic), phases (resident)
                                   or rounds of four phases (naive) */
     int64_t tested;            /* point tests made: a point is tested in a phase of its parity only
                                   if a neighbour moved since its last test (all points in the first
